@@ -113,7 +113,12 @@ typedef struct {
                             conditional while nodes repeat chunks of fused iterations until
                             no system is active, the active list and counts rebuilt on the
                             device after every chunk (no host check inside the loop); with
-                            profile = 1 one loop in four runs as with 1.  1: each chunk of
+                            profile = 1 one loop in four runs as with 1.  Where one
+                            thread-block cluster can hold a system's vectors (tile = -1,
+                            stencil radius 4 or 6, from 1,536 points on), one kernel runs all
+                            iterations of a system instead -- of every system, or on grids
+                            that need clusters of 8 or 16 blocks of the last active ones.
+                            1: each chunk of
                             fused iterations is a captured graph replayed by the host, which
                             reads the active count after every chunk.  0: the kernels are
                             launched one by one */
@@ -158,7 +163,9 @@ typedef struct {
   /* with options.profile: per COCG kernel class (0 projector dots, 1 H apply (matvec),
    * 2 scalar steps, 3 x/r update, 4 direction update) the summed event time, the number
    * of launches, and the algorithmic bytes moved (active systems x grid points x bytes per
-   * point; projector data and scalars not counted).  Slots 5 and 6 of kernel_seconds: the
+   * point; projector data and scalars not counted).  A launch of the resident kernel counts in
+   * class 1, with ten vector passes per system and iteration (what the launched kernels of an
+   * iteration move; it keeps most of them in shared memory).  Slots 5 and 6 of kernel_seconds: the
    * time of the sampled chunks whose launches covered at most 32 systems (the tail) and
    * more (the bulk); slots 5 and 6 of kernel_launches: those chunks' iterations */
   double kernel_seconds[8];
@@ -167,8 +174,10 @@ typedef struct {
   int precision_bytes;     /* bytes of one real value in the COCG vectors (4 or 8) */
   int tile_rows;           /* tiling the H-apply kernel used for launches over many systems:
                               0 = 32 x 8 column tiles, -2 = 64 x 8 two-point tiles, h > 0 =
-                              full-row tiles of height h */
-  int tile_rows_tail;      /* the same for launches over at most 32 systems */
+                              full-row tiles of height h, -7 = the resident kernel (one
+                              thread-block cluster runs the whole COCG loop of a system) */
+  int tile_rows_tail;      /* the same for launches over at most 32 systems, or for the last
+                              active systems (-7) */
   long long nonconv_solves;   /* solves that ended above the tolerance (iteration cap, or
                                  refinement rounds or restarts used up) */
   long long breakdown_solves; /* solves that broke down (p^T A p = 0 or non-finite) */

@@ -23,6 +23,7 @@
 #include "checkpoint.cuh"
 #include "cocg.cuh"
 #include "cocg_fused.cuh"
+#include "cocg_resident.cuh"
 #include "small.cuh"
 
 using namespace rpa;
@@ -118,6 +119,17 @@ struct rpa_ctx {
   DevBuf loopctl_d;
   long long loop_no = 0;
   int prof_cpx_bytes = 0;
+  // resident COCG (cocg_resident.cu) per COCG precision (FP32, FP64) and cluster size 2^i:
+  // shape (known once asked for) and projector tables (built on first use, dropped with the
+  // projectors); h_*: the internal projector groups on the host
+  struct ResidentPlan {
+    bool known = false, tables = false;
+    rpa::ResidentShape sh;
+    rpa::DevBuf roff, rstep, gslot, gchi, goff, groups, lwarp, lkey, lchi, gmask;
+  };
+  ResidentPlan resident[2][5];
+  std::vector<int> h_goff, h_gidx;
+  std::vector<double> h_gchi;
   // non-fatal outcome of the current call (results are still written): RPA_ENOCONV or
   // RPA_EBREAKDOWN (the more severe is kept), with its reason
   rpa_status soft = RPA_OK;
@@ -710,10 +722,12 @@ static rpa_status run_chunk_graph(rpa_ctx* c, const CocgView<T>& cv, const Fused
 // long as more than W_{i+1} are active.  After every chunk the active list and counts are
 // rebuilt on the device and a one-thread kernel sets the level's condition.  An iteration
 // counter bounds every level (the per-system cap marks every system by maxit + 2 chunks),
-// so each loop ends even if no status changes.  Graphs are cached like the chunk graphs.
+// so each loop ends even if no status changes.  Graphs are cached like the chunk graphs.  With
+// stop > 0 the last level ends once at most `stop` systems are active (at a chunk's end: their
+// latest direction is in p_in, their beta in sysd).
 template <typename T>
 static rpa_status run_loop_graph(rpa_ctx* c, const CocgView<T>& cv, const FusedBufs<T>& fb,
-                                 int maxit, int ty_bulk, int ty_tail) {
+                                 int maxit, int ty_bulk, int ty_tail, int stop = 0) {
   const int nsys = cv.nsys;
   int w0 = 1;
   while (w0 < fb.nact) w0 <<= 1;
@@ -722,10 +736,10 @@ static rpa_status run_loop_graph(rpa_ctx* c, const CocgView<T>& cv, const FusedB
   {
     int w = 1;
     while (w < w0) w <<= 1;
-    for (w >>= 1; w >= 1; w >>= 1) widths.push_back(w);
+    for (w >>= 1; w >= 1 && w > stop; w >>= 1) widths.push_back(w);
   }
   struct Key {
-    int kind, tsize, maxit, w0, ty_bulk, ty_tail;
+    int kind, tsize, maxit, w0, ty_bulk, ty_tail, stop;
     double tol;
     CocgView<T> cv;
     FusedBufs<T> fb;
@@ -737,6 +751,7 @@ static rpa_status run_loop_graph(rpa_ctx* c, const CocgView<T>& cv, const FusedB
   k.w0 = w0;
   k.ty_bulk = ty_bulk;
   k.ty_tail = ty_tail;
+  k.stop = stop;
   k.tol = c->opt.stern_tol;
   k.cv = cv;
   k.fb = fb;
@@ -811,7 +826,7 @@ static rpa_status run_loop_graph(rpa_ctx* c, const CocgView<T>& cv, const FusedB
       }, &tail);
     parent_launches = (int)(rpa_kernel_launches(c) - l0);
     for (size_t i = 0; i < widths.size() && err == cudaSuccess; ++i) {
-      const int wnext = i + 1 < widths.size() ? widths[i + 1] : 0;
+      const int wnext = i + 1 < widths.size() ? widths[i + 1] : stop;
       // the prologue's iterations are counted by the first level's check
       const int add = i == 0 ? kChunkIters : 0;
       cudaGraphConditionalHandle h;
@@ -862,6 +877,197 @@ static rpa_status run_loop_graph(rpa_ctx* c, const CocgView<T>& cv, const FusedB
   return RPA_OK;
 }
 
+// Projector tables of a resident plan: the internal groups' entries by block of the cluster.
+template <typename T>
+static rpa_status resident_tables(rpa_ctx* c, rpa_ctx::ResidentPlan& pl) {
+  const ResidentShape& sh = pl.sh;
+  const int nx = c->grid.n[0], ny = c->grid.n[1], nz = c->grid.n[2], G = sh.G;
+  const int ng = c->ngroup;
+  // owner brick of every y and z coordinate, and its extents
+  std::vector<int> ry(ny), rz(nz), y0(sh.gy + 1), z0(sh.gz + 1);
+  for (int q = 0; q <= sh.gy; ++q) y0[q] = (int)((long long)q * ny / sh.gy);
+  for (int q = 0; q <= sh.gz; ++q) z0[q] = (int)((long long)q * nz / sh.gz);
+  for (int q = 0; q < sh.gy; ++q)
+    for (int y = y0[q]; y < y0[q + 1]; ++y) ry[y] = q;
+  for (int q = 0; q < sh.gz; ++q)
+    for (int z = z0[q]; z < z0[q + 1]; ++z) rz[z] = q;
+  struct Entry {
+    int layer, slot, group;
+    long long e;
+  };
+  std::vector<std::vector<Entry>> grp(G);
+  std::vector<std::vector<unsigned char>> cnt(G, std::vector<unsigned char>(65536, 0));
+  std::vector<unsigned> mask(std::max(ng, 1), 0u);
+  for (int g = 0; g < ng; ++g)
+    for (int e = c->h_goff[g]; e < c->h_goff[g + 1]; ++e) {
+      const int q = c->h_gidx[e], x = q % nx, y = q / nx % ny, z = q / (nx * ny);
+      const int rank = ry[y] + sh.gy * rz[z];
+      const int by = y0[ry[y] + 1] - y0[ry[y]];
+      const int slot = ((z - z0[rz[z]]) * by + (y - y0[ry[y]])) * sh.pitch + x;
+      const int l = cnt[rank][slot];
+      if (l == 255) {  // more groups at a point than the layers count: the launched iteration
+        pl.sh.G = 0;
+        return RPA_OK;
+      }
+      cnt[rank][slot]++;
+      grp[rank].push_back({l, slot, g, e});
+      mask[g] |= 1u << rank;
+    }
+  const int nw = sh.threads / 32;
+  std::vector<int> roff(1, 0), rstep(1, 0), goff(1, 0), groups, lwarp(1, 0);
+  std::vector<unsigned short> gslot;
+  std::vector<unsigned> lkey;
+  std::vector<T> gchi, lchi;
+  auto put = [&](std::vector<T>& v, long long e) {
+    for (int l = 0; l < kProjChunk; ++l)
+      v.push_back(e < 0 ? (T)0 : (T)c->h_gchi[(size_t)e * kProjChunk + l]);
+  };
+  for (int r = 0; r < G; ++r) {
+    std::vector<Entry>& v = grp[r];
+    for (size_t i = 0; i < v.size();) {  // entries of a group are consecutive
+      size_t j = i;
+      while (j < v.size() && v[j].group == v[i].group) ++j;
+      groups.push_back(v[i].group);
+      groups.push_back((int)rstep.size() - 1 - roff.back());
+      while (i < j) {
+        const size_t end = std::min(j, i + 32 * res_steps<T>());
+        for (; i < end; i += 32)
+          for (size_t l = i; l < i + 32; ++l) {
+            gslot.push_back(l < end ? (unsigned short)v[l].slot : 0);
+            put(gchi, l < end ? v[l].e : -1);
+          }
+        i = end;
+        rstep.push_back((int)gslot.size() / 32);
+      }
+      groups.push_back((int)rstep.size() - 1 - roff.back());
+    }
+    goff.push_back((int)groups.size() / 3);
+    roff.push_back((int)rstep.size() - 1);
+    if ((roff[r + 1] - roff[r]) * kProjChunk > sh.bym * sh.bzm * sh.pitch) {
+      pl.sh.G = 0;  // the records' sums share the space of w
+      return RPA_OK;
+    }
+    // runs of slots with about the same number of entries, by layer
+    std::sort(v.begin(), v.end(), [](const Entry& a, const Entry& b) {
+      return a.slot != b.slot ? a.slot < b.slot : a.layer < b.layer;
+    });
+    size_t i = 0;
+    for (int w = 0; w < nw; ++w) {
+      size_t j = w + 1 == nw ? v.size() : std::max(i, v.size() * (size_t)(w + 1) / nw);
+      while (j > i && j < v.size() && v[j].slot == v[j - 1].slot) ++j;
+      std::sort(v.begin() + i, v.begin() + j, [](const Entry& a, const Entry& b) {
+        return a.layer != b.layer ? a.layer < b.layer : a.slot < b.slot;
+      });
+      while (i < j) {
+        const int layer = v[i].layer;
+        for (int l = 0; l < 32; ++l) {
+          const bool in = i < j && v[i].layer == layer;
+          lkey.push_back(in ? (unsigned)v[i].group << 16 | (unsigned)v[i].slot : ~0u);
+          put(lchi, in ? v[i].e : -1);
+          if (in) ++i;
+        }
+      }
+      lwarp.push_back((int)lkey.size() / 32);
+    }
+  }
+  auto up = [&](DevBuf& b, const void* p, size_t bytes) -> rpa_status {
+    CK(b.ensure(std::max<size_t>(bytes, 16)));
+    if (bytes) CK(cudaMemcpyAsync(b.p, p, bytes, cudaMemcpyHostToDevice, c->stream));
+    return RPA_OK;
+  };
+  CKS(up(pl.roff, roff.data(), roff.size() * sizeof(int)));
+  CKS(up(pl.rstep, rstep.data(), rstep.size() * sizeof(int)));
+  CKS(up(pl.gslot, gslot.data(), gslot.size() * sizeof(unsigned short)));
+  CKS(up(pl.gchi, gchi.data(), gchi.size() * sizeof(T)));
+  CKS(up(pl.goff, goff.data(), goff.size() * sizeof(int)));
+  CKS(up(pl.groups, groups.data(), groups.size() * sizeof(int)));
+  CKS(up(pl.lwarp, lwarp.data(), lwarp.size() * sizeof(int)));
+  CKS(up(pl.lkey, lkey.data(), lkey.size() * sizeof(unsigned)));
+  CKS(up(pl.lchi, lchi.data(), lchi.size() * sizeof(T)));
+  CKS(up(pl.gmask, mask.data(), mask.size() * sizeof(unsigned)));
+  CK(cudaStreamSynchronize(c->stream));  // the host arrays go away
+  pl.tables = true;
+  return RPA_OK;
+}
+
+// Smaller grids keep the captured loop: the rule starts below the smallest grid it was measured
+// on (12^3: one probe-point of 20 Lanczos steps in FP64, 144 -> 55 ms).
+constexpr long long kResidentMinPoints = 1536;
+
+// The cluster size for nsys systems, or no plan where the resident kernel does not apply: an
+// explicit tiling or loop mode asks for the launched iteration.
+template <typename T>
+static rpa_status resident_plan(rpa_ctx* c, int nsys, rpa_ctx::ResidentPlan** out) {
+  *out = nullptr;
+  if (c->opt.tile != -1 || c->opt.graphs != 2 || c->nd < kResidentMinPoints ||
+      !resident_supported(c->grid.fd_radius))
+    return RPA_OK;
+  const int k = sizeof(T) == 4 ? 0 : 1;
+  rpa_ctx::ResidentPlan* best = nullptr;
+  // the fewest blocks whose memory holds p and w: a brick then has the least halo and the
+  // fewest barriers per point; with fewer systems than blocks fit, larger clusters use the rest
+  for (int i = 0; i < 5; ++i) {
+    rpa_ctx::ResidentPlan& pl = c->resident[k][i];
+    if (!pl.known) {
+      CK(resident_shape<T>(c->grid.n[0], c->grid.n[1], c->grid.n[2], c->grid.fd_radius, c->ngroup,
+                           1 << i, &pl.sh));
+      pl.known = true;
+    }
+    if (pl.sh.G == 0) continue;
+    if (!best || nsys <= pl.sh.clusters) best = &pl;
+  }
+  if (!best) return RPA_OK;
+  if (!best->tables) CKS(resident_tables<T>(c, *best));
+  if (best->sh.G) *out = best;
+  return RPA_OK;
+}
+
+template <typename T>
+static rpa_status resident_loop(rpa_ctx* c, const CocgView<T>& cv, rpa_ctx::ResidentPlan& pl,
+                                int maxit, bool cont) {
+  ResidentProj<T> pj;
+  pj.ngroup = c->ngroup;
+  pj.coef = opd<T>(c).coef.template as<T>();
+  pj.roff = pl.roff.as<int>();
+  pj.rstep = pl.rstep.as<int>();
+  pj.gslot = pl.gslot.as<unsigned short>();
+  pj.gchi = pl.gchi.as<T>();
+  pj.goff = pl.goff.as<int>();
+  pj.groups = pl.groups.as<int>();
+  pj.lwarp = pl.lwarp.as<int>();
+  pj.lkey = pl.lkey.as<unsigned>();
+  pj.lchi = pl.lchi.as<T>();
+  pj.gmask = pl.gmask.as<unsigned>();
+  const bool prof = c->opt.profile && c->have_pev && c->prof_stats;
+  long long iters = 0;
+  auto count = [&](int sign) -> rpa_status {  // iterations of all systems so far
+    std::vector<int> si((size_t)cv.nsys * kSysI);
+    CK(cudaMemcpyAsync(si.data(), cv.sysi, sizeof(int) * si.size(), cudaMemcpyDeviceToHost,
+                       c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+    for (int s = 0; s < cv.nsys; ++s)
+      if (si[(size_t)s * kSysI + kStatus] != kIdle) iters += sign * si[(size_t)s * kSysI + kIters];
+    return RPA_OK;
+  };
+  if (prof) {
+    CKS(count(-1));
+    CK(cudaEventRecord(c->pev[0], c->stream));
+  }
+  CK(resident_cocg<T>(cv, pl.sh, pj, c->p2.as<cpx<T>>(), maxit, cont ? 1 : 0, c->stream));
+  if (prof) {
+    CK(cudaEventRecord(c->pev[1], c->stream));
+    CKS(count(1));
+    float ms = 0.f;
+    CK(cudaEventElapsedTime(&ms, c->pev[0], c->pev[1]));
+    rpa_stats* st = c->prof_stats;
+    st->kernel_seconds[1] += 1e-3 * ms;
+    st->kernel_launches[1] += 1;
+    st->kernel_bytes[1] += 10.0 * sizeof(cpx<T>) * (double)iters * (double)c->nd;
+    st->precision_bytes = (int)(sizeof(cpx<T>) / 2);
+  }
+  return RPA_OK;
+}
+
 // COCG iterations until no system is active.  Expects r (and x) set for the active systems;
 // forms the projector coefficients of r, then iterates the fused kernels.  With cont, the
 // recurrence continues from the direction kept in p (and its projector coefficients in cp)
@@ -869,11 +1075,38 @@ static rpa_status run_loop_graph(rpa_ctx* c, const CocgView<T>& cv, const FusedB
 template <typename T>
 static rpa_status cocg_loop(rpa_ctx* c, const CocgView<T>& cv_all, int maxit, bool cont = false) {
   int cnt[kNumStatus];
+  rpa_ctx::ResidentPlan* pl = nullptr;
+  CKS(resident_plan<T>(c, cv_all.nsys, &pl));
+  // Launched iterations until at most `tail` systems are active, the resident kernel from there
+  // on.  Up to four blocks per system it wins at any number of systems (26^3, 320 systems: 24
+  // against 44 ms per chi0; 27 x 25 x 53: 70 against 109 ms).  Larger clusters leave SMs idle
+  // (15 clusters of 8, 7 of 16 on 152 SMs) and move more halo per point, and launches over
+  // hundreds of systems are faster per system; the crossing was measured at about 8 systems
+  // per cluster (52^3, 1,280 systems: 393 ms launched throughout, 389 resident throughout, 369 /
+  // 360 / 349 / 346 ms handing over at 1 / 2 / 4 / 8 per cluster).  FP64 is bound by the FP64
+  // pipe, which clusters of 16 use on 112 of the SMs only: two systems per cluster there.
+  int tail = 0;
+  if (pl) {
+    const bool whole = sizeof(T) == 8 ? pl->sh.G <= 8 : pl->sh.G <= 4;
+    if (!whole) {
+      tail = 1;
+      while (tail < (sizeof(T) == 8 ? 2 : 8) * pl->sh.clusters) tail *= 2;
+      CKS(counts(c, cv_all.nsys, cnt, false));
+    }
+    if (whole || cnt[kActive] <= tail) {
+      if (c->prof_stats) c->prof_stats->tile_rows = c->prof_stats->tile_rows_tail = kTileResident;
+      return resident_loop<T>(c, cv_all, *pl, maxit, cont);
+    }
+  }
   int done_iters = 0;
   const bool prof = c->opt.profile && c->have_pev && c->prof_stats;
   FusedBufs<T> fb = make_fused<T>(c);
   CK(proj_dots<T>(cv_all.nl, cv_all.nd, cv_all.nsys, cv_all.r, cv_all.sysi, 1 << kActive, fb.cr,
                   c->stream));
+  // the resident kernel keeps no projector coefficients of the direction: form them anew
+  if (cont && pl)
+    CK(proj_dots<T>(cv_all.nl, cv_all.nd, cv_all.nsys, cv_all.p, cv_all.sysi, 1 << kActive, fb.cp,
+                    c->stream));
   CK(fused_prepare<T>(cv_all, fb, c->stream, cont ? 0 : 1));
   if (cont) fb.first = 0;
   // launches cover only the active systems, listed at every chunk boundary
@@ -885,13 +1118,15 @@ static rpa_status cocg_loop(rpa_ctx* c, const CocgView<T>& cv_all, int maxit, bo
   if (fb.nact > 0) CKS(choose_tiling<T>(c, cv, fb, &ty_bulk, &ty_tail));
   if (c->prof_stats) {
     c->prof_stats->tile_rows = ty_bulk;
-    c->prof_stats->tile_rows_tail = ty_tail;
+    c->prof_stats->tile_rows_tail = tail ? kTileResident : ty_tail;
   }
   const bool graphs = c->opt.graphs != 0;
   // graphs = 2: the whole loop on the device; with profiling, every kProfLoopEvery-th loop
   // runs host-checked instead, its sample chunks timed with events
-  if (c->opt.graphs == 2 && fb.nact > 0 && !(prof && c->loop_no++ % kProfLoopEvery == 0))
-    return run_loop_graph<T>(c, cv, fb, maxit, ty_bulk, ty_tail);
+  if (c->opt.graphs == 2 && fb.nact > 0 && !(prof && c->loop_no++ % kProfLoopEvery == 0)) {
+    CKS(run_loop_graph<T>(c, cv, fb, maxit, ty_bulk, ty_tail, tail));
+    return tail ? resident_loop<T>(c, cv_all, *pl, maxit, true) : RPA_OK;
+  }
   const size_t cpxb = sizeof(cpx<T>);
   int chunk_no = 0;
   while (fb.nact > 0) {
@@ -949,6 +1184,7 @@ static rpa_status cocg_loop(rpa_ctx* c, const CocgView<T>& cv_all, int maxit, bo
       st->precision_bytes = (int)(cpxb / 2);
     }
     fb.nact = cnt[kActive];
+    if (tail && fb.nact <= tail) return resident_loop<T>(c, cv_all, *pl, maxit, true);
     if (done_iters > maxit + 2 * kChunkIters) break;  // every system is marked by then
   }
   return RPA_OK;
@@ -1927,6 +2163,11 @@ rpa_status rpa_set_projectors(rpa_ctx* c, int ngroups, const int* nnz, const int
     CK(cudaMemcpy(c->coef_lo.p, gcoef_lo.data(), sizeof(float) * NG * kProjChunk, cudaMemcpyHostToDevice));
   }
   c->ngroup = NG;
+  c->h_goff = goff;
+  c->h_gidx = gidx;
+  c->h_gchi = gchi;
+  for (auto& row : c->resident)  // the number of groups sets the shapes' shared memory
+    for (auto& pl : row) pl.known = pl.tables = false;
   // host copy of the inputs, for lane contexts
   long long nidx = 0, nchi = 0, ngam = 0;
   for (int g = 0; g < ngroups; ++g) {
