@@ -266,7 +266,27 @@ __device__ __forceinline__ void seg_sums(typename Val<T>::V (&acc)[L],
   }
 }
 
-// warps take (segment, 32 lines) units in turn, so that a segment's edges are uniform in a warp
+// Unit u of a warp: its lane's segment and line.  FP32: a warp takes 32 lines of one segment,
+// so that the segment's edges are uniform in it.  FP64: segments and lines are dealt to the
+// lanes without gaps -- an FP64 instruction occupies its pipe for 64 cycles whatever the number
+// of lanes that need it, and a small brick has few lines.
+template <typename T>
+__device__ __forceinline__ int units_of(int lines, int segs) {
+  return sizeof(T) == 8 ? (lines * segs + 31) >> 5 : ((lines + 31) >> 5) * segs;
+}
+template <typename T>
+__device__ __forceinline__ bool unit(int u, int lane, int lines, int segs, int& seg, int& line) {
+  if (sizeof(T) == 8) {
+    const int v = u * 32 + lane;
+    seg = v / lines;
+    line = v - seg * lines;
+    return seg < segs;
+  }
+  const int lw = (lines + 31) >> 5;
+  seg = u / lw;
+  line = (u - seg * lw) * 32 + lane;
+  return line < lines;
+}
 __device__ __forceinline__ int warp_id() { return __shfl_sync(0xffffffffu, tid() >> 5, 0); }
 
 // Segments of L outputs of a line of b points, evenly spread, the first at 0 and the last at
@@ -289,16 +309,17 @@ __device__ __noinline__ void part_x() {
   typename Val<T>::K c[R + 1];
 #pragma unroll
   for (int m = 1; m <= R; ++m) c[m] = k.kc[m];
-  const int nx = k.nx, pitch = k.pitch, nrow = k.by * k.bz, nrw = (nrow + 31) >> 5, per = k.px;
+  const int nx = k.nx, pitch = k.pitch, nrow = k.by * k.bz, per = k.px;
   const Segs sg(nx, L);
+  const int units = units_of<T>(nrow, sg.n);
   const V* const P = smem_vec<T>(0);
   V* const W = smem_vec<T>(k.off_w());
   const int lane = tid() & 31, nw = blockDim.x >> 5;
 #pragma unroll 1
-  for (int u = warp_id(); u < nrw * sg.n; u += nw) {
-    const int seg = u / nrw, row = (u - seg * nrw) * 32 + lane;
+  for (int u = warp_id(); u < units; u += nw) {
+    int seg, row;
+    if (!unit<T>(u, lane, nrow, sg.n, seg, row)) continue;
     const int i0 = sg.start(seg), keep = (seg + 1 < sg.n ? sg.start(seg + 1) : nx) - i0;
-    if (row >= nrow) continue;
     const V* const p = P + row * pitch + i0;
     V v[L + 2 * R];
     // R points to the left and to the right: of the row, of its other end, or zeros; wl, wr:
@@ -410,20 +431,21 @@ __device__ __noinline__ void part_z() {
   typename Val<T>::K c[R + 1];
 #pragma unroll
   for (int m = 1; m <= R; ++m) c[m] = k.kc[2 * (kMaxRadius + 1) + m];
-  const int nx = k.nx, by = k.by, pitch = k.pitch, ncol = nx * by, ncw = (ncol + 31) >> 5;
+  const int nx = k.nx, by = k.by, pitch = k.pitch, ncol = nx * by;
   const int stride = by * pitch, plane = nx * k.ny;
   const unsigned mg_nx = k.a.mg_nx;
   const Axis ax{k.z0, k.bz, k.nz, k.pz};
   const Segs sg(ax.b, L);
+  const int units = units_of<T>(ncol, sg.n);
   const V* const P = smem_vec<T>(0);
   V* const W = smem_vec<T>(k.off_w());
   const V* const pg = k.pg + nx * k.y0;
   const int lane = tid() & 31, nw = blockDim.x >> 5;
 #pragma unroll 1
-  for (int u = warp_id(); u < ncw * sg.n; u += nw) {
-    const int seg = u / ncw, col = (u - seg * ncw) * 32 + lane;
+  for (int u = warp_id(); u < units; u += nw) {
+    int seg, col;
+    if (!unit<T>(u, lane, ncol, sg.n, seg, col)) continue;
     const int i0 = sg.start(seg), keep = (seg + 1 < sg.n ? sg.start(seg + 1) : ax.b) - i0;
-    if (col >= ncol) continue;
     const int yl = quot(col, mg_nx), base = yl * (pitch - nx) + col;  // yl * pitch + x
     V v[L + 2 * R];
     line_load<T, L, R>(v, P + base, stride, pg + col, plane, i0, ax);
@@ -449,11 +471,12 @@ __device__ __noinline__ cpx<T> part_y() {
   typename Val<T>::K c[R + 1];
 #pragma unroll
   for (int m = 1; m <= R; ++m) c[m] = k.kc[kMaxRadius + 1 + m];
-  const int nx = k.nx, pitch = k.pitch, ncol = nx * k.bz, ncw = (ncol + 31) >> 5;
+  const int nx = k.nx, pitch = k.pitch, ncol = nx * k.bz;
   const int plane = nx * k.ny, zstep = k.by * pitch;
   const unsigned mg_nx = k.a.mg_nx;
   const Axis ax{k.y0, k.by, k.ny, k.py};
   const Segs sg(ax.b, L);
+  const int units = units_of<T>(ncol, sg.n);
   const V* const P = smem_vec<T>(0);
   V* const W = smem_vec<T>(k.off_w());
   const V* const pg = k.pg + plane * k.z0;
@@ -462,10 +485,10 @@ __device__ __noinline__ cpx<T> part_y() {
   V sum = vzero<T>();
   const int lane = tid() & 31, nw = blockDim.x >> 5;
 #pragma unroll 1
-  for (int u = warp_id(); u < ncw * sg.n; u += nw) {
-    const int seg = u / ncw, col = (u - seg * ncw) * 32 + lane;
+  for (int u = warp_id(); u < units; u += nw) {
+    int seg, col;
+    if (!unit<T>(u, lane, ncol, sg.n, seg, col)) continue;
     const int i0 = sg.start(seg), keep = (seg + 1 < sg.n ? sg.start(seg + 1) : ax.b) - i0;
-    if (col >= ncol) continue;
     const int zl = quot(col, mg_nx), x = col - zl * nx;
     const int base = zl * zstep + x, gl = zl * plane + x;
     T vl[L];
@@ -559,7 +582,9 @@ __device__ __forceinline__ void read_totals(const typename Acc<T>::A* slots, int
 
 #define RES_BY_LEN(l, call) \
   switch (l) {              \
+    case 1: if constexpr (sizeof(T) == 8) call(1); break; \
     case 2: call(2); break; \
+    case 3: if constexpr (sizeof(T) == 8) call(3); break; \
     case 4: call(4); break; \
     case 5: call(5); break; \
     case 6: if constexpr (sizeof(T) == 4) call(6); break; \
@@ -1036,7 +1061,7 @@ __global__ void __launch_bounds__(max_threads<T>(), 1) k_cocg_resident(const __g
 }
 
 // ---- shapes ----------------------------------------------------------------------------
-constexpr int kLens[] = {2, 4, 5, 6, 7};
+constexpr int kLens[] = {1, 2, 3, 4, 5, 6, 7};
 
 // segment length of one axis: `lines` lines of `b` points on `warps` warps, N = FP work of an
 // output next to the loads of an input
@@ -1044,12 +1069,14 @@ int seg_len(int bmin, int b, int lines, int warps, int R, bool fp64, double* cos
   int best = 2;
   *cost = 1e300;
   for (int L : kLens) {
-    if (L > bmin || (fp64 && L > 5)) continue;  // a segment lies inside the smallest brick
-    const long long w = (long long)((lines + 31) / 32) * ((b + L - 1) / L);
+    // a segment lies inside the smallest brick; lengths built: 1 - 5 (FP64), 2, 4 - 7
+    if (L > bmin || (fp64 ? L > 5 : L == 1 || L == 3)) continue;
+    const long long segs = (b + L - 1) / L;
+    const long long w = fp64 ? ((long long)lines * segs + 31) / 32 : (long long)((lines + 31) / 32) * segs;
     const double rounds = (double)((w + warps - 1) / warps);
     // FP64 arithmetic keeps its pipe busy whatever the number of warps: count the warps'
     // instructions; FP32 counts the rounds of the block
-    const double c = fp64 ? (double)w * (24.0 * L + 0.5 * (L + 2 * R)) / 4.0 + rounds * 2.0
+    const double c = fp64 ? std::ceil(w / 4.0) * (24.0 * L + 0.5 * (L + 2 * R)) + rounds * 2.0
                           : rounds * (24.0 * L / 2 + 2.0 * (L + 2 * R) + 20.0);
     if (c < *cost) {
       *cost = c;
