@@ -81,7 +81,10 @@ struct rpa_ctx {
   DevBuf tile_roff, tile_ranges;  // per 1-D COCG tile: (group, entry range) lists
   DevBuf lam[3];
   // interpolation operators (transposed, coarse x fine) per axis
-  DevBuf interpWt[3], cnodes_d[3];
+  DevBuf interpWt[3], interpTi[3], interpTw[3], cnodes_d[3];
+  // interpolation workspace: coarse and fine arrays of calls on host data, the two
+  // intermediate arrays, partial sums and E_c
+  DevBuf itco, itfi, it1, it2, itpart, itec;
   std::vector<long long> cnodes[3];
   int interp_built = -1, stride_built[3] = {0, 0, 0};
   // wave workspace
@@ -1823,6 +1826,11 @@ static rpa_status build_interp(rpa_ctx* c) {
     CK(c->interpWt[a].ensure(sizeof(double) * (size_t)m * n));
     CK(interp_matrix(n, m, c->grid.bc[a], k, c->cnodes_d[a].as<long long>(),
                      c->interpWt[a].as<double>(), c->stream));
+    CK(c->interpTi[a].ensure(sizeof(int4) * n));
+    CK(c->interpTw[a].ensure(sizeof(double) * 4 * n));
+    if (k != RPA_INTERP_FOURIER)
+      CK(interp_taps(n, m, c->interpWt[a].as<double>(), c->interpTi[a].as<int4>(),
+                     c->interpTw[a].as<double>(), c->stream));
   }
   CK(cudaStreamSynchronize(c->stream));
   c->interp_built = kind;
@@ -1836,33 +1844,49 @@ static long long num_probes(rpa_ctx* c) {
   return P;
 }
 
-// d_coarse (device, nw x P) -> d_fine (device, nw x N_d) and E_c (device scalar)
+// d_coarse (device, nw x P) -> d_fine (device, nw x N_d) and E_c (device scalar); queued on the
+// context's stream.  d_coarse is read only by the first of the passes, d_fine written by the last.
 static rpa_status interpolate_dev(rpa_ctx* c, const double* dco, double* dfi, double* ec_dev) {
   CKS(build_interp(c));
   const int m[3] = {(int)c->cnodes[0].size(), (int)c->cnodes[1].size(), (int)c->cnodes[2].size()};
   const int* n = c->grid.n;
   const long long P = (long long)m[0] * m[1] * m[2];
-  DevBuf t1, t2, part;
-  CK(t1.ensure(sizeof(double) * c->nw * (long long)n[0] * m[1] * m[2]));
-  CK(t2.ensure(sizeof(double) * c->nw * (long long)n[0] * n[1] * m[2]));
+  DevBuf &t1 = c->it1, &t2 = c->it2, &part = c->itpart;
+  const long long p1 = (long long)n[0] * m[1] * m[2], p2 = (long long)n[0] * n[1] * m[2];
+  CK(t1.ensure(sizeof(double) * c->nw * p1));
+  CK(t2.ensure(sizeof(double) * c->nw * p2));
+  if (c->opt.interp != RPA_INTERP_FOURIER) {
+    // four taps per axis; the sums for E_c come with the last pass
+    const int nblk = taps_blocks(c->nd);
+    CK(part.ensure(sizeof(double) * nblk * c->nw));
+    CK(taps_product(dco, P, t1.as<double>(), p1, c->interpTi[0].as<int4>(),
+                    c->interpTw[0].as<double>(), 1, m[0], n[0], (long long)m[1] * m[2], c->nw,
+                    nullptr, nullptr, c->stream));
+    CK(taps_product(t1.as<double>(), p1, t2.as<double>(), p2, c->interpTi[1].as<int4>(),
+                    c->interpTw[1].as<double>(), n[0], m[1], n[1], m[2], c->nw, nullptr, nullptr,
+                    c->stream));
+    CK(taps_product(t2.as<double>(), p2, dfi, c->nd, c->interpTi[2].as<int4>(),
+                    c->interpTw[2].as<double>(), (long long)n[0] * n[1], m[2], n[2], 1, c->nw,
+                    c->weight_d.as<double>(), part.as<double>(), c->stream));
+    CK(ec_final(nblk * c->nw, part.as<double>(), ec_dev, c->stream));
+    return RPA_OK;
+  }
   int d0[3] = {m[0], m[1], m[2]};
-  CK((mode_product<double, double, double>(dco, P, t1.as<double>(), (long long)n[0] * m[1] * m[2],
+  CK((mode_product<double, double, double>(dco, P, t1.as<double>(), p1,
                                            c->interpWt[0].as<double>(), 0, d0, n[0], c->nw,
                                            nullptr, c->stream)));
   int d1[3] = {n[0], m[1], m[2]};
-  CK((mode_product<double, double, double>(t1.as<double>(), (long long)n[0] * m[1] * m[2],
-                                           t2.as<double>(), (long long)n[0] * n[1] * m[2],
+  CK((mode_product<double, double, double>(t1.as<double>(), p1, t2.as<double>(), p2,
                                            c->interpWt[1].as<double>(), 1, d1, n[1], c->nw,
                                            nullptr, c->stream)));
   int d2[3] = {n[0], n[1], m[2]};
-  CK((mode_product<double, double, double>(t2.as<double>(), (long long)n[0] * n[1] * m[2], dfi,
-                                           c->nd, c->interpWt[2].as<double>(), 2, d2, n[2],
-                                           c->nw, nullptr, c->stream)));
+  CK((mode_product<double, double, double>(t2.as<double>(), p2, dfi, c->nd,
+                                           c->interpWt[2].as<double>(), 2, d2, n[2], c->nw,
+                                           nullptr, c->stream)));
   const int nblk = (int)std::max<long long>(1, std::min<long long>(256, (c->nd + 1023) / 1024));
   CK(part.ensure(sizeof(double) * nblk * c->nw));
   CK(ec_reduce(c->nd, c->nw, dfi, c->weight_d.as<double>(), part.as<double>(), nblk, ec_dev,
                c->stream));
-  CK(cudaStreamSynchronize(c->stream));
   return RPA_OK;
 }
 
@@ -2387,14 +2411,23 @@ rpa_status rpa_interpolate(rpa_ctx* c, const double* d_coarse, double* d_fine, d
   if (!c->have_freq) return fail(c, RPA_ESTATE, "no frequencies set");
   CK(cudaSetDevice(c->device));
   const long long P = num_probes(c);
-  DevBuf dco, dfi, ecd;
-  CK(dco.ensure(sizeof(double) * c->nw * P));
-  CK(dfi.ensure(sizeof(double) * c->nw * c->nd));
-  CK(ecd.ensure(sizeof(double)));
-  CKS(copy_in(c, dco.p, d_coarse, sizeof(double) * c->nw * P, where));
-  CKS(interpolate_dev(c, dco.as<double>(), dfi.as<double>(), ecd.as<double>()));
-  if (d_fine) CKS(copy_out(c, d_fine, dfi.p, sizeof(double) * c->nw * c->nd, where));
-  if (ec) CKS(copy_out(c, ec, ecd.p, sizeof(double), where));
+  const bool dev = where == RPA_DEVICE;
+  CK(c->itec.ensure(sizeof(double)));
+  double* fine = d_fine;
+  const double* coarse = d_coarse;
+  if (!dev) {
+    CK(c->itco.ensure(sizeof(double) * c->nw * P));
+    CKS(copy_in(c, c->itco.p, d_coarse, sizeof(double) * c->nw * P, where));
+    coarse = c->itco.as<double>();
+  }
+  if (!dev || !d_fine) {
+    CK(c->itfi.ensure(sizeof(double) * c->nw * c->nd));
+    fine = c->itfi.as<double>();
+  }
+  double* ecd = dev && ec ? ec : c->itec.as<double>();
+  CKS(interpolate_dev(c, coarse, fine, ecd));
+  if (!dev && d_fine) CKS(copy_out(c, d_fine, fine, sizeof(double) * c->nw * c->nd, where));
+  if (!dev && ec) CKS(copy_out(c, ec, ecd, sizeof(double), where));
   CK(cudaStreamSynchronize(c->stream));
   return RPA_OK;
 }

@@ -223,18 +223,124 @@ __global__ void k_ec_partial(long long nd, int nw, const double* __restrict__ df
   }
 }
 
-__global__ void k_ec_final(int n, const double* __restrict__ part, double* __restrict__ ec) {
-  if (threadIdx.x != 0) return;
+// One block: 256 strided sums in order, then a tree (a single thread took 71 us for 1,370
+// partial sums, one FP64 addition of 64 cycles after the other; 4 us now).
+__global__ void __launch_bounds__(256) k_ec_final(int n, const double* __restrict__ part,
+                                                  double* __restrict__ ec) {
   double t = 0.0;
-  for (int i = 0; i < n; ++i) t += part[i];
-  ec[0] = t / (2.0 * 3.14159265358979323846);
+  for (int i = threadIdx.x; i < n; i += 256) t += part[i];
+  __shared__ double sh[8];
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = t;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    t = 0.0;
+    for (int w = 0; w < 8; ++w) t += sh[w];
+    ec[0] = t / (2.0 * 3.14159265358979323846);
+  }
+}
+
+// The at most four nonzero weights of each fine point (trilinear, tricubic and identity
+// operators), coarse indices ascending; unused ones repeat the last index with weight 0.
+__global__ void k_interp_taps(int n, int m, const double* __restrict__ Wt, int4* __restrict__ ti,
+                              double* __restrict__ tw) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  int id[4] = {0, 0, 0, 0}, cnt = 0;
+  double w[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int j = 0; j < m; ++j) {
+    const double v = Wt[(long long)j * n + i];
+    if (v == 0.0) continue;
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+      if (t == cnt) {
+        id[t] = j;
+        w[t] = v;
+      }
+    ++cnt;
+  }
+#pragma unroll
+  for (int t = 1; t < 4; ++t)
+    if (t >= cnt) id[t] = id[t - 1];
+  ti[i] = make_int4(id[0], id[1], id[2], id[3]);
+  for (int t = 0; t < 4; ++t) tw[4 * i + t] = w[t];
+}
+
+cudaError_t interp_taps(int n, int m, const double* Wt, int4* ti, double* tw, cudaStream_t s) {
+  k_interp_taps<<<(n + 127) / 128, 128, 0, s>>>(n, m, Wt, ti, tw);
+  note_launch();
+  return cudaGetLastError();
+}
+
+// Interpolation along one axis by the taps: out[i2][a][i0] = sum_t w_t(a) in[i2][ti_t(a)][i0],
+// i0 < inner, a < nout, and with part the block's sum of the outputs times weight[b].  Bound by
+// the FP64 pipe (4 multiply-adds per output of the last axis, 19 us for ten 52^3 arrays); the
+// dense mode product did one per coarse node, 26 of them, nearly all with weight 0: 125 us.
+constexpr int kTapOut = 4;  // outputs per thread
+__global__ void __launch_bounds__(256) k_taps(const double* __restrict__ in, long long in_bs,
+                                              double* __restrict__ out, long long out_bs,
+                                              const int4* __restrict__ ti,
+                                              const double* __restrict__ tw, unsigned inner,
+                                              unsigned nin, unsigned nout, unsigned per,
+                                              const double* __restrict__ weight,
+                                              double* __restrict__ part) {
+  in += (long long)blockIdx.y * in_bs;
+  out += (long long)blockIdx.y * out_bs;
+  double sum = 0.0;
+#pragma unroll
+  for (int u = 0; u < kTapOut; ++u) {
+    const unsigned o = (blockIdx.x * kTapOut + u) * 256 + threadIdx.x;
+    if (o < per) {
+      const unsigned t = o / inner, i0 = o - t * inner, i2 = t / nout, a = t - i2 * nout;
+      const double* src = in + (size_t)i2 * nin * inner + i0;
+      const int4 id = ti[a];
+      const double2 w0 = reinterpret_cast<const double2*>(tw)[2 * a],
+                    w1 = reinterpret_cast<const double2*>(tw)[2 * a + 1];
+      double v = w0.x * src[(size_t)id.x * inner];
+      v += w0.y * src[(size_t)id.y * inner];
+      v += w1.x * src[(size_t)id.z * inner];
+      v += w1.y * src[(size_t)id.w * inner];
+      out[o] = v;
+      sum += v;
+    }
+  }
+  if (!part) return;
+  __shared__ double sh[8];
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = sum;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    sum = 0.0;
+    for (int w = 0; w < 8; ++w) sum += sh[w];
+    part[(long long)blockIdx.y * gridDim.x + blockIdx.x] = sum * weight[blockIdx.y];
+  }
+}
+
+int taps_blocks(long long per) { return (int)((per + 256 * kTapOut - 1) / (256 * kTapOut)); }
+
+cudaError_t taps_product(const double* in, long long in_bs, double* out, long long out_bs,
+                         const int4* ti, const double* tw, long long inner, int nin, int nout,
+                         long long outer, int batch, const double* weight, double* part,
+                         cudaStream_t s) {
+  const long long per = inner * nout * outer;
+  k_taps<<<dim3(taps_blocks(per), batch), 256, 0, s>>>(in, in_bs, out, out_bs, ti, tw,
+                                                       (unsigned)inner, (unsigned)nin,
+                                                       (unsigned)nout, (unsigned)per, weight, part);
+  note_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t ec_final(int n, const double* part, double* ec, cudaStream_t s) {
+  k_ec_final<<<1, 256, 0, s>>>(n, part, ec);
+  note_launch();
+  return cudaGetLastError();
 }
 
 cudaError_t ec_reduce(long long nd, int nw, const double* dfine, const double* weight,
                       double* part, int nblk, double* ec, cudaStream_t s) {
   dim3 g(nblk, nw);
   k_ec_partial<<<g, 256, 0, s>>>(nd, nw, dfine, weight, part);
-  k_ec_final<<<1, 32, 0, s>>>(nblk * nw, part, ec);
+  k_ec_final<<<1, 256, 0, s>>>(nblk * nw, part, ec);
   note_launch(2);
   return cudaGetLastError();
 }
