@@ -1,6 +1,6 @@
 // True residual r = b - (H - sigma) x of the Sternheimer systems (Eq. 4) with
 // b_n = -psi_n (.) u, in the 2.5-D blocked form of the fused COCG kernels: a block owns a
-// 32 x 8 column tile, walks z with the 2R+1 values of its column in registers and the current
+// column tile (see tile_of), walks z with the 2R+1 values of its column in registers and the current
 // xy plane (with an R-wide halo) in shared memory, next plane prefetched.  Used for the
 // initial residual of every solve, the true-residual recheck of the FP64 form and the FP64
 // residual of each refinement round of the mixed form (T = double, low-precision copies of r
@@ -16,6 +16,7 @@
 // the projector terms, b and the sums stay in FP64.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "cocg.cuh"
@@ -25,7 +26,12 @@ namespace rpa {
 
 namespace {
 
-constexpr int kRTX = 32, kRTY = 8;
+constexpr int kRThreads = 256;
+// halo points a thread loads per plane
+template <int R>
+__host__ __device__ constexpr int halo_per_thread() {
+  return R <= 6 ? 3 : 4;
+}
 
 // the stencil coefficients as double-float pairs (kernel parameters)
 struct DfCoef {
@@ -38,11 +44,11 @@ struct DfCoef {
 // DF (with XDF): the whole residual in double-float arithmetic on the FP32 units; without
 // DF the loaded pairs are summed into FP64 and the FP64 arithmetic follows.
 template <typename T, typename TL, int R, bool SMEM_CD, bool DF>
-__global__ void __launch_bounds__(kRTX * kRTY, sizeof(T) == 4 ? 3 : 2)
+__global__ void __launch_bounds__(kRThreads, sizeof(T) == 4 ? 3 : 2)
     k_resid_fused(CocgView<T> cv, const cpx<T>* __restrict__ x, cpx<T>* __restrict__ r,
                   cpx<T>* __restrict__ pdir, int mask, cpx<TL>* __restrict__ r_lo,
                   cpx<TL>* __restrict__ p_lo, cpx<TL>* __restrict__ x_lo, int zchunk,
-                  DfCoef dc, const cpx<TL>* __restrict__ p_keep, DfAux aux) {
+                  int tx, int ty, DfCoef dc, const cpx<TL>* __restrict__ p_keep, DfAux aux) {
   constexpr bool XDF = sizeof(T) == 8 && std::is_same<TL, float>::value;
   static_assert(!DF || XDF, "the double-float path is the mixed form's refinement");
   using V = typename std::conditional<DF, cdf, cpx<T>>::type;  // stored neighbour values
@@ -57,22 +63,24 @@ __global__ void __launch_bounds__(kRTX * kRTY, sizeof(T) == 4 ? 3 : 2)
     const int ran = cv.sysi[(long long)s * kSysI + kIters] - cv.sysi[(long long)s * kSysI + kIterBase];
     pmode = ran <= 0 ? 0 : ((ran & 1) ? 2 : 1);
   }
-  constexpr int EXN = kRTX + 2 * R, EYN = kRTY + 2 * R;
-  constexpr int PLN = EXN * EYN;
-  constexpr int NHALO = PLN - kRTX * kRTY;
-  constexpr int HPT = (NHALO + kRTX * kRTY - 1) / (kRTX * kRTY);
-  __shared__ V pl[2 * PLN];
+  // tile of tx x ty points (see tile_of), one per thread; two planes with R points around it
+  // (the stencil is a star: the corners are not loaded), then the projector coefficients
+  constexpr int HPT = halo_per_thread<R>();
+  const int EXN = tx + 2 * R, PLN = EXN * (ty + 2 * R), NHALO = 2 * R * (tx + ty);
   __shared__ AT sh[8 * 4];
   extern __shared__ __align__(16) unsigned char dyn_smem[];
+  V* const pl = reinterpret_cast<V*>(dyn_smem);
+  unsigned char* const cd_smem = dyn_smem + 2 * sizeof(V) * PLN;
   const Stencil<T>& st = cv.st;
   const int nx = st.nx, ny = st.ny, nz = st.nz;
   const int plane = nx * ny;
-  const int ntx = (nx + kRTX - 1) / kRTX;
-  const int tx0 = (blockIdx.x % ntx) * kRTX, ty0 = (blockIdx.x / ntx) * kRTY;
+  const int ntx = (nx + tx - 1) / tx;
+  const int tx0 = (blockIdx.x % ntx) * tx, ty0 = (blockIdx.x / ntx) * ty;
   const int z0 = blockIdx.z * zchunk, z1 = min(z0 + zchunk, nz);
-  const int lx = threadIdx.x & (kRTX - 1), ly = threadIdx.x / kRTX;
+  const bool own = (int)threadIdx.x < tx * ty;
+  const int ly = threadIdx.x / tx, lx = threadIdx.x - ly * tx;
   const int gx = tx0 + lx, gy = ty0 + ly;
-  const bool valid = gx < nx && gy < ny;
+  const bool valid = own && gx < nx && gy < ny;
   const long long sbase = (long long)s * cv.nd;
   const cpx<T>* __restrict__ xs = x + sbase;
   const float4* __restrict__ xd = reinterpret_cast<const float4*>(x) + sbase;  // XDF
@@ -86,11 +94,11 @@ __global__ void __launch_bounds__(kRTX * kRTY, sizeof(T) == 4 ? 3 : 2)
   const cdf* cdd = nullptr;  // DF: the coefficients as double-float pairs in shared memory
   if (SMEM_CD) {
     if constexpr (DF) {
-      cdf* scd = reinterpret_cast<cdf*>(dyn_smem);
+      cdf* scd = reinterpret_cast<cdf*>(cd_smem);
       for (int i = threadIdx.x; i < ncd; i += blockDim.x) scd[i] = cdf_of(cd[i]);
       cdd = scd;
     } else {
-      cpx<T>* scd = reinterpret_cast<cpx<T>*>(dyn_smem);
+      cpx<T>* scd = reinterpret_cast<cpx<T>*>(cd_smem);
       for (int i = threadIdx.x; i < ncd; i += blockDim.x) scd[i] = cd[i];
       cd = scd;  // read after the first barrier of the z loop
     }
@@ -104,29 +112,26 @@ __global__ void __launch_bounds__(kRTX * kRTY, sizeof(T) == 4 ? 3 : 2)
   int own_xy;
   {
     const int xx = wrap_or_neg(gx, nx, st.bcx), yy = wrap_or_neg(gy, ny, st.bcy);
-    own_xy = (xx < 0 || yy < 0) ? -1 : xx + nx * yy;
+    own_xy = (!own || xx < 0 || yy < 0) ? -1 : xx + nx * yy;
   }
   int halo_xy[HPT], halo_slot[HPT];
 #pragma unroll
   for (int k = 0; k < HPT; ++k) {
-    const int hi = threadIdx.x + k * kRTX * kRTY;
+    const int hi = threadIdx.x + k * blockDim.x;
     halo_slot[k] = -1;
     halo_xy[k] = -1;
     if (hi < NHALO) {
-      // R rows above, the 2R padding points of each tile row, R rows below
+      // R rows above and below the tile, then the 2R points beside each of its rows
       int ey, ex;
-      if (hi < R * EXN) {
-        ey = hi / EXN;
-        ex = hi - ey * EXN;
-      } else if (hi < R * EXN + kRTY * 2 * R) {
-        const int t = hi - R * EXN;
-        ey = R + t / (2 * R);
-        const int c = t - (ey - R) * 2 * R;
-        ex = (c < R) ? c : kRTX + c;
+      if (hi < 2 * R * tx) {
+        const int row = hi / tx;
+        ey = row < R ? row : ty + row;
+        ex = R + hi - row * tx;
       } else {
-        const int t = hi - R * EXN - kRTY * 2 * R;
-        ey = R + kRTY + t / EXN;
-        ex = t - (ey - R - kRTY) * EXN;
+        const int t = hi - 2 * R * tx;
+        const int row = t / (2 * R), c = t - row * 2 * R;
+        ey = R + row;
+        ex = c < R ? c : tx + c;
       }
       halo_slot[k] = ey * EXN + ex;
       const int xx = wrap_or_neg(tx0 - R + ex, nx, st.bcx),
@@ -182,7 +187,7 @@ __global__ void __launch_bounds__(kRTX * kRTY, sizeof(T) == 4 ? 3 : 2)
   for (int z = z0; z < z1; ++z) {
     const int bo = ((z - z0) & 1) * PLN;
     zq[2 * R] = nq;
-    pl[bo + own_slot] = zq[R];
+    if (own) pl[bo + own_slot] = zq[R];
 #pragma unroll
     for (int k = 0; k < HPT; ++k)
       if (halo_slot[k] >= 0) pl[bo + halo_slot[k]] = hv[k];
@@ -293,17 +298,50 @@ __global__ void __launch_bounds__(kRTX * kRTY, sizeof(T) == 4 ? 3 : 2)
   }
 }
 
+// Tile of the xy plane: the shape that keeps the most of its threads on grid points.  32 x 8
+// tiles leave 38 % of them idle on a 40-point row, 34 % on a 26^2 plane; full or half rows of
+// 40, 26 or 52 points do not.  Bound by the FP32 pipe (about 1,300 instructions per point in
+// double-float arithmetic): the residual of 2,048 systems on 40^3, 12.8 ms with 32 x 8 tiles, 8.8 ms
+// with 40 x 6.
+struct Tile {
+  int tx, ty, n;
+};
+template <int R>
+Tile tile_of(int nx, int ny, int nz_chunks, int max_tiles, size_t value) {
+  Tile best{32, 8, ((nx + 31) / 32) * ((ny + 7) / 8)};
+  double best_cost = 1e300;
+  for (int parts = 0; parts <= 64; ++parts) {
+    const int tx = parts == 0 ? 32 : (nx + parts - 1) / parts;
+    if (tx < 4 || tx > 64) continue;
+    for (int ty = std::min(kRThreads / tx, ny + 7); ty >= 2; --ty) {
+      const int thr = (tx * ty + 31) / 32 * 32;
+      if (2 * R * (tx + ty) > halo_per_thread<R>() * thr) continue;
+      if (2 * value * (tx + 2 * R) * (ty + 2 * R) > 40 * 1024) continue;
+      const long long n = (long long)((nx + tx - 1) / tx) * ((ny + ty - 1) / ty);
+      if (n * nz_chunks > max_tiles) continue;
+      // warps per plane, each with its share of the halo loads
+      const double cost = (double)n * (thr / 32) * (1.0 + 0.08 * 2 * R * (tx + ty) / thr);
+      if (cost < best_cost) {
+        best_cost = cost;
+        best = Tile{tx, ty, (int)n};
+      }
+    }
+  }
+  return best;
+}
+
 template <typename T, typename TL, int R>
 void launch_r(const CocgView<T>& cv, const cpx<T>* x, cpx<T>* r, cpx<T>* pdir, int mask,
               cpx<TL>* r_lo, cpx<TL>* p_lo, cpx<TL>* x_lo, bool use_df,
               const cpx<TL>* p_keep, const DfAux& aux, cudaStream_t s) {
-  constexpr size_t kPlanes = 2 * sizeof(cpx<T>) * (kRTX + 2 * R) * (kRTY + 2 * R);
-  size_t cdb = sizeof(cpx<T>) * cv.nl.ngroup * kProjChunk;
-  if (cdb + kPlanes + 1024 > 48 * 1024) cdb = 0;
   const int nx = cv.st.nx, ny = cv.st.ny, nz = cv.st.nz;
-  const int zchunk = nz <= 64 ? nz : 32;
-  const dim3 grid(((nx + kRTX - 1) / kRTX) * ((ny + kRTY - 1) / kRTY), cv.nsys,
-                  (nz + zchunk - 1) / zchunk);
+  const int zchunk = nz <= 64 ? nz : 32, nzc = (nz + zchunk - 1) / zchunk;
+  const Tile t = tile_of<R>(nx, ny, nzc, cv.tiles, sizeof(cpx<T>));
+  const size_t planes = 2 * sizeof(cpx<T>) * (t.tx + 2 * R) * (t.ty + 2 * R);
+  size_t cdb = sizeof(cpx<T>) * cv.nl.ngroup * kProjChunk;
+  if (cdb + planes + 1024 > 48 * 1024) cdb = 0;
+  const int thr = (t.tx * t.ty + 31) / 32 * 32;
+  const dim3 grid(t.n, cv.nsys, nzc);
   DfCoef dc{};
   if (use_df && sizeof(T) == 8) {  // hi + lo splits of the neighbour coefficients
     for (int m = 0; m <= R; ++m) {
@@ -321,20 +359,20 @@ void launch_r(const CocgView<T>& cv, const cpx<T>* x, cpx<T>* r, cpx<T>* pdir, i
   if constexpr (sizeof(T) == 8 && std::is_same<TL, float>::value) {
     if (use_df) {
       if (cdb)
-        k_resid_fused<T, TL, R, true, true><<<grid, kRTX * kRTY, cdb, s>>>(
-            cv, x, r, pdir, mask, r_lo, p_lo, x_lo, zchunk, dc, p_keep, aux);
+        k_resid_fused<T, TL, R, true, true><<<grid, thr, planes + cdb, s>>>(
+            cv, x, r, pdir, mask, r_lo, p_lo, x_lo, zchunk, t.tx, t.ty, dc, p_keep, aux);
       else
-        k_resid_fused<T, TL, R, false, true><<<grid, kRTX * kRTY, 0, s>>>(
-            cv, x, r, pdir, mask, r_lo, p_lo, x_lo, zchunk, dc, p_keep, aux);
+        k_resid_fused<T, TL, R, false, true><<<grid, thr, planes, s>>>(
+            cv, x, r, pdir, mask, r_lo, p_lo, x_lo, zchunk, t.tx, t.ty, dc, p_keep, aux);
       return;
     }
   }
   if (cdb)
-    k_resid_fused<T, TL, R, true, false><<<grid, kRTX * kRTY, cdb, s>>>(
-        cv, x, r, pdir, mask, r_lo, p_lo, x_lo, zchunk, dc, p_keep, aux);
+    k_resid_fused<T, TL, R, true, false><<<grid, thr, planes + cdb, s>>>(
+        cv, x, r, pdir, mask, r_lo, p_lo, x_lo, zchunk, t.tx, t.ty, dc, p_keep, aux);
   else
-    k_resid_fused<T, TL, R, false, false><<<grid, kRTX * kRTY, 0, s>>>(
-        cv, x, r, pdir, mask, r_lo, p_lo, x_lo, zchunk, dc, p_keep, aux);
+    k_resid_fused<T, TL, R, false, false><<<grid, thr, planes, s>>>(
+        cv, x, r, pdir, mask, r_lo, p_lo, x_lo, zchunk, t.tx, t.ty, dc, p_keep, aux);
 }
 
 }  // namespace
@@ -351,8 +389,7 @@ cudaError_t cocg_resid(const CocgView<T>& cv, const cpx<T>* x, cpx<T>* r, cpx<T>
   const DfAux& ax = aux ? *aux : noaux;
   const int nx = cv.st.nx, ny = cv.st.ny, nz = cv.st.nz;
   const int zchunk = nz <= 64 ? nz : 32;
-  const long long used = (long long)((nx + kRTX - 1) / kRTX) * ((ny + kRTY - 1) / kRTY) *
-                         ((nz + zchunk - 1) / zchunk);
+  const long long used = (long long)((nx + 31) / 32) * ((ny + 7) / 8) * ((nz + zchunk - 1) / zchunk);
   if (used > cv.tiles) return cudaErrorInvalidValue;  // partial buffer too small
   switch (cv.st.R) {
     case 1: launch_r<T, TL, 1>(cv, x, r, pdir, mask, r_lo, p_lo, x_lo, use_df, p_keep, ax, s); break;
