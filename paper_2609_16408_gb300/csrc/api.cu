@@ -380,6 +380,15 @@ static int gram_chunks(long long nd) {
   return (int)std::max<long long>(1, std::min<long long>(256, (nd + 4095) / 4096));
 }
 
+// FP64 form: more chunks (of at least 96 points) while the tiles of nb probe-points would leave
+// the GPU idle
+static int gram_chunks64(long long nd, int ns, int nb) {
+  const int ts = ns <= 8 ? 8 : 16, nt = (ns + ts - 1) / ts;
+  const long long tiles = (long long)nb * nt * (nt + 1) / 2;
+  const long long want = std::min<long long>((nd + 95) / 96, (608 + tiles - 1) / tiles);
+  return (int)std::min<long long>(256, std::max<long long>(gram_chunks(nd), want));
+}
+
 static size_t per_probe_bytes(const rpa_ctx* c) {
   const long long nd = c->nd, ns = c->ns;
   size_t b = (size_t)ns * nd * cpx_bytes(c) * 4;
@@ -436,7 +445,12 @@ static rpa_status ensure_workspace(rpa_ctx* c, int nb) {
   CK(c->part.ensure(sizeof(double) * S * part_stride(c) * 4));
   CK(c->sysd.ensure(sizeof(double) * S * kSysD));
   CK(c->sysi.ensure(sizeof(int) * S * kSysI));
-  CK(c->gpart.ensure(sizeof(double) * nb * gram_chunks(nd) * c->ns * c->ns));
+  // a wave may hold fewer probe-points than nb, with more chunks each
+  size_t gchunks = (size_t)nb * gram_chunks(nd);
+  if (c->opt.precision == RPA_FP64)
+    for (int b = 1; b <= nb; ++b)
+      gchunks = std::max(gchunks, (size_t)b * gram_chunks64(nd, c->ns, b));
+  CK(c->gpart.ensure(sizeof(double) * gchunks * c->ns * c->ns));
   CK(c->cmat.ensure(cb * nb * c->ns * c->ns));
   CK(c->probe_d.ensure(sizeof(long long) * nb));
   CK(c->pomega_d.ensure(sizeof(double) * nb));
@@ -1204,7 +1218,7 @@ static rpa_status solve_fp64(rpa_ctx* c, int nb, const double* u, const int* act
   CocgView<double> cv = make_view<double>(c, nb, u, x, r, p, w);
   CK(galerkin_guess<double>(c->nd, c->ns, nb, c->d64.psi.as<double>(), c->eps_d.as<double>(),
                             c->pomega_d.as<double>(), u, active, c->dV, c->gpart.as<double>(),
-                            gram_chunks(c->nd), c->cmat.as<cpx<double>>(), x, c->stream));
+                            gram_chunks64(c->nd, c->ns, nb), c->cmat.as<cpx<double>>(), x, c->stream));
   CK(set_status(S, c->ns, active, kActive, c->sysi.as<int>(), c->stream));
   CK(proj_dots<double>(cv.nl, c->nd, S, x, cv.sysi, 1 << kActive, cv.cdot, c->stream));
   CK((cocg_resid<double, double>(cv, x, r, p, 1 << kActive, nullptr, nullptr, nullptr,

@@ -11,23 +11,34 @@ namespace rpa {
 // -------------------------------------------------------------------------------------------
 // Galerkin projection
 // -------------------------------------------------------------------------------------------
-// gpart[b][c][k][n] = sum_{r in chunk c} psi_k(r) psi_n(r) u_b(r)
-template <typename T>
+// gpart[b][c][k][n] = sum_{r in chunk c} psi_k(r) psi_n(r) u_b(r), symmetric in k and n: only
+// the tiles on and above the diagonal are formed, and mirrored.  Bound by the FP64 pipe; tiles of
+// TS = 8 or 16 states waste less of it on padding and on the diagonal than 32 (8 states on
+// 12^3, one probe-point: one block of a 32-tile, 484 us; 8-tiles over 18 chunks, 6 us).  The 256 threads are 256 / (TS/2)^2 groups that take the
+// rows of a stage in turn, 2 x 2 outputs per thread.
+template <typename T, int TS>
 __global__ void __launch_bounds__(256) k_gram(long long nd, int ns, const T* __restrict__ psi,
                                               const T* __restrict__ u,
                                               const int* __restrict__ active, int nchunk,
                                               long long chunk_len, double* __restrict__ gpart) {
-  constexpr int TS = 32, RK = 32;
+  constexpr int RK = 32, H = TS / 2, GROUPS = 256 / (H * H);
   __shared__ T sA[RK][TS + 1];
   __shared__ T sB[RK][TS + 1];
+  __shared__ T sum[GROUPS > 1 ? 256 * 4 : 1];
+  int kt = 0, ntl = blockIdx.x;  // tile (kt, ntl), kt <= ntl, from the row-wise index
   const int nt = (ns + TS - 1) / TS;
-  const int kt = blockIdx.x / nt, ntl = blockIdx.x - kt * nt;
+  while (ntl >= nt - kt) {
+    ntl -= nt - kt;
+    ++kt;
+  }
+  ntl += kt;
   const int b = blockIdx.y, c = blockIdx.z;
   if (active && !active[b]) return;
   const int k0 = kt * TS, n0 = ntl * TS;
   const long long r0 = (long long)c * chunk_len;
   const long long r1 = min(r0 + chunk_len, nd);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const int grp = threadIdx.x / (H * H), q = threadIdx.x - grp * (H * H);
+  const int tx = q % H, ty = q / H;
   const T* ub = u + (long long)b * nd;
   T acc[2][2] = {{0, 0}, {0, 0}};
   for (long long rb = r0; rb < r1; rb += RK) {
@@ -40,8 +51,8 @@ __global__ void __launch_bounds__(256) k_gram(long long nd, int ns, const T* __r
       sB[rr][kk] = (okr && n < ns) ? psi[(long long)n * nd + r] * ub[r] : (T)0;
     }
     __syncthreads();
-#pragma unroll 8
-    for (int rr = 0; rr < RK; ++rr) {
+#pragma unroll 2
+    for (int rr = grp; rr < RK; rr += GROUPS) {
       const T a0 = sA[rr][2 * ty], a1 = sA[rr][2 * ty + 1];
       const T b0 = sB[rr][2 * tx], b1 = sB[rr][2 * tx + 1];
       acc[0][0] += a0 * b0;
@@ -51,13 +62,28 @@ __global__ void __launch_bounds__(256) k_gram(long long nd, int ns, const T* __r
     }
     __syncthreads();
   }
+  if (GROUPS > 1) {  // the groups' sums in order
+#pragma unroll
+    for (int i = 0; i < 4; ++i) sum[i * 256 + threadIdx.x] = acc[i >> 1][i & 1];
+    __syncthreads();
+    if (grp > 0) return;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      T t = 0;
+      for (int g = 0; g < GROUPS; ++g) t += sum[i * 256 + g * (H * H) + q];
+      acc[i >> 1][i & 1] = t;
+    }
+  }
   double* out = gpart + ((long long)b * nchunk + c) * ns * ns;
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
       const int k = k0 + 2 * ty + i, n = n0 + 2 * tx + j;
-      if (k < ns && n < ns) out[(long long)k * ns + n] = (double)acc[i][j];
+      if (k < ns && n < ns) {
+        out[(long long)k * ns + n] = (double)acc[i][j];
+        if (kt != ntl) out[(long long)n * ns + k] = (double)acc[i][j];
+      }
     }
 }
 
@@ -83,15 +109,16 @@ __global__ void k_gram_coef(int ns, int nchunk, const double* __restrict__ gpart
   cmat[(long long)b * ns * ns + e] = cv;
 }
 
-// x0[(b,n)][r] = sum_k psi_k(r) C_b[k][n]; output tile 64 points x 32 states for one b.
-// Point tiles run along gridDim.x (up to 2^31 - 1 tiles), (b, state tile) along gridDim.y.
-template <typename T>
+// x0[(b,n)][r] = sum_k psi_k(r) C_b[k][n]; output tile of TN states (the least that holds ns, up
+// to 32: padding costs FP64 time like states) x 2048 / TN points for one b.  Point tiles run
+// along gridDim.x (up to 2^31 - 1 tiles), (b, state tile) along gridDim.y.
+template <typename T, int TN>
 __global__ void __launch_bounds__(256) k_x0(long long nd, int ns, int nb,
                                             const T* __restrict__ psi,
                                             const cpx<T>* __restrict__ cmat,
                                             const int* __restrict__ active,
                                             cpx<T>* __restrict__ x0) {
-  constexpr int TR = 64, TN = 32, KK = 16;
+  constexpr int TR = 2048 / TN, KK = 16, NT = TN / 2, NR = 256 / NT;
   __shared__ T sP[KK][TR];
   __shared__ cpx<T> sC[KK][TN];
   const int ntn = (ns + TN - 1) / TN;
@@ -99,7 +126,7 @@ __global__ void __launch_bounds__(256) k_x0(long long nd, int ns, int nb,
   if (active && !active[b]) return;
   const long long r0 = (long long)blockIdx.x * TR;
   const int n0 = nt * TN;
-  const int tr = threadIdx.x & 15, tn = threadIdx.x >> 4;  // 4 points x 2 states per thread
+  const int tr = threadIdx.x % NR, tn = threadIdx.x / NR;  // 4 points x 2 states per thread
   cpx<T> acc[4][2];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
@@ -122,7 +149,7 @@ __global__ void __launch_bounds__(256) k_x0(long long nd, int ns, int nb,
     for (int kk = 0; kk < KK; ++kk) {
       T pv[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) pv[i] = sP[kk][tr + 16 * i];
+      for (int i = 0; i < 4; ++i) pv[i] = sP[kk][tr + NR * i];
       const cpx<T> c0 = sC[kk][2 * tn], c1 = sC[kk][2 * tn + 1];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -134,7 +161,7 @@ __global__ void __launch_bounds__(256) k_x0(long long nd, int ns, int nb,
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const long long r = r0 + tr + 16 * i;
+    const long long r = r0 + tr + NR * i;
     if (r >= nd) continue;
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
@@ -149,14 +176,24 @@ cudaError_t galerkin_guess(long long nd, int ns, int nb, const T* psi, const dou
                            const double* omega, const T* u, const int* probe_active, double dV,
                            double* gpart, int nchunk, cpx<T>* cmat, cpx<T>* x0, cudaStream_t s) {
   const long long chunk_len = (nd + nchunk - 1) / nchunk;
-  const int nt = (ns + 31) / 32;
-  dim3 g1(nt * nt, nb, nchunk);
-  k_gram<T><<<g1, 256, 0, s>>>(nd, ns, psi, u, probe_active, nchunk, chunk_len, gpart);
+  const int ts = ns <= 8 ? 8 : 16, nt = (ns + ts - 1) / ts;
+  dim3 g1(nt * (nt + 1) / 2, nb, nchunk);
+  if (ts == 8)
+    k_gram<T, 8><<<g1, 256, 0, s>>>(nd, ns, psi, u, probe_active, nchunk, chunk_len, gpart);
+  else
+    k_gram<T, 16><<<g1, 256, 0, s>>>(nd, ns, psi, u, probe_active, nchunk, chunk_len, gpart);
   dim3 g2((ns * ns + 255) / 256, nb);
   k_gram_coef<T><<<g2, 256, 0, s>>>(ns, nchunk, gpart, eps, omega, probe_active, dV, cmat);
   if ((long long)nb * ((ns + 31) / 32) > 65535) return cudaErrorInvalidValue;
-  dim3 g3((unsigned)((nd + 63) / 64), nb * ((ns + 31) / 32));
-  k_x0<T><<<g3, 256, 0, s>>>(nd, ns, nb, psi, cmat, probe_active, x0);
+  auto grid = [&](int tn) {
+    return dim3((unsigned)((nd + 2048 / tn - 1) / (2048 / tn)), nb * ((ns + tn - 1) / tn));
+  };
+  if (ns <= 8)
+    k_x0<T, 8><<<grid(8), 256, 0, s>>>(nd, ns, nb, psi, cmat, probe_active, x0);
+  else if (ns <= 16)
+    k_x0<T, 16><<<grid(16), 256, 0, s>>>(nd, ns, nb, psi, cmat, probe_active, x0);
+  else
+    k_x0<T, 32><<<grid(32), 256, 0, s>>>(nd, ns, nb, psi, cmat, probe_active, x0);
   note_launch(3);
   return cudaGetLastError();
 }
