@@ -164,6 +164,10 @@ __device__ __forceinline__ double acc_xor(double v, int o) { return __shfl_xor_s
 __device__ __forceinline__ df acc_xor(df v, int o) {
   return df{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
 }
+__device__ __forceinline__ double acc_lane(double v, int l) { return __shfl_sync(0xffffffffu, v, l); }
+__device__ __forceinline__ df acc_lane(df v, int l) {
+  return df{__shfl_sync(0xffffffffu, v.hi, l), __shfl_sync(0xffffffffu, v.lo, l)};
+}
 __device__ __forceinline__ double acc_val(double v) { return v; }
 __device__ __forceinline__ double acc_val(df v) { return df_val(v); }
 __device__ __forceinline__ void acc_from(double& a, double v) { a = v; }
@@ -517,7 +521,7 @@ __device__ __noinline__ cpx<T> part_y() {
         if constexpr (sizeof(T) == 4)
           wv = kfma(cfma(acc[i], c0 + vl[i], -om, pc), mkk(-eps), pc);
         else
-          wv = cfma(acc[i], (c0 + vl[i]) - eps, -om, pc);
+          wv = cfma(acc[i], vl[i] + (c0 - eps), -om, pc);
         w[i * pitch] = wv;
         T pr, pi;
         parts(pc, pr, pi);
@@ -549,12 +553,16 @@ __device__ __forceinline__ void block_total(T (&v)[NQ], T* red, typename Acc<T>:
   if ((lane & (32 / NQ - 1)) == 0) red[wid * NQ + q] = v[0];
   __syncthreads();
   if (wid == 0) {
+    // warp 0 holds value q of warps w, w + 32 / NQ in lane q * (32 / NQ) + w: one addition and
+    // one tree for all values together (FP64 additions take 64 cycles of the pipe each)
+    constexpr int S = 32 / NQ;
+    const int qq = lane / S, w = lane % S;
+    typename Acc<T>::A t = acc_of(w < nw ? red[w * NQ + qq] : (T)0);
+    if (nw > S) t = acc_add(t, acc_of(w + S < nw ? red[(w + S) * NQ + qq] : (T)0));
 #pragma unroll
-    for (int i = 0; i < NQ; ++i) {
-      out[i] = acc_of(lane < nw ? red[lane * NQ + i] : (T)0);
+    for (int x = S / 2; x > 0; x >>= 1) t = acc_add(t, acc_xor(t, x));
 #pragma unroll
-      for (int s = 16; s > 0; s >>= 1) out[i] = acc_add(out[i], acc_xor(out[i], s));
-    }
+    for (int i = 0; i < NQ; ++i) out[i] = acc_lane(t, i * S);
   }
 }
 
@@ -572,12 +580,14 @@ __device__ __forceinline__ void post_totals(cg::cluster_group& cl, const A (&v)[
 template <typename T, int NQ>
 __device__ __forceinline__ void read_totals(const typename Acc<T>::A* slots, int G,
                                             typename Acc<T>::A (&v)[NQ]) {
-  const int lane = threadIdx.x & 31;
+  // value q of blocks r, r + 32 / NQ in lane q * (32 / NQ) + r
+  constexpr int S = 32 / NQ;
+  const int lane = threadIdx.x & 31, q = lane / S, r = lane % S;
+  typename Acc<T>::A t = r < G ? slots[r * 4 + q] : acc_of((T)0);
+  if (G > S) t = acc_add(t, r + S < G ? slots[(r + S) * 4 + q] : acc_of((T)0));
+  for (int x = 1; x < G && x < S; x <<= 1) t = acc_add(t, acc_xor(t, x));
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) {
-    v[q] = lane < G ? slots[lane * 4 + q] : acc_of((T)0);
-    for (int o = 1; o < G; o <<= 1) v[q] = acc_add(v[q], acc_xor(v[q], o));
-  }
+  for (int i = 0; i < NQ; ++i) v[i] = acc_lane(t, i * S);
 }
 
 #define RES_BY_LEN(l, call) \
@@ -826,9 +836,15 @@ __device__ __noinline__ Sum3<T> phase_update() {
       stg2(xg + g, x);
     T re, im;
     parts(r, re, im);
-    s0 += re * re + im * im;
-    s1 += re * re - im * im;
-    s2 += (T)2 * re * im;
+    if constexpr (sizeof(T) == 8) {  // three multiply-adds; combined at the end
+      s0 = fma(re, re, s0);
+      s1 = fma(im, im, s1);
+      s2 = fma(re, im, s2);
+    } else {
+      s0 += re * re + im * im;
+      s1 += re * re - im * im;
+      s2 += (T)2 * re * im;
+    }
   };
   int i0 = tid();
 #pragma unroll 1
@@ -853,6 +869,7 @@ __device__ __noinline__ Sum3<T> phase_update() {
     locate(i0, mg, nx, pad, rowoff, slot, g);
     step(slot, g, RRES ? rs[slot] : ldg2(rg + g), XRES ? xs[slot] : ldg2(xg + g), W[slot], P[slot]);
   }
+  if constexpr (sizeof(T) == 8) return Sum3<T>{{s0 + s1, s0 - s1, 2 * s2}};
   return Sum3<T>{{s0, s1, s2}};
 }
 
