@@ -69,6 +69,33 @@ __device__ __forceinline__ void put_split(uint8_t* hi, uint8_t* lo, uint32_t off
   *reinterpret_cast<float*>(lo + off) = umma::to_tf32(v - h);
 }
 
+// four K-adjacent values of one row: a whole 16-byte core-matrix row of each part, so that
+// eight lanes with eight rows write 128 contiguous bytes (one value per lane along K hits one
+// bank eight times)
+__device__ __forceinline__ void put_split4(uint8_t* hi, uint8_t* lo, uint32_t off, float4 v) {
+  float4 h, l;
+  h.x = umma::to_tf32(v.x);
+  h.y = umma::to_tf32(v.y);
+  h.z = umma::to_tf32(v.z);
+  h.w = umma::to_tf32(v.w);
+  l.x = umma::to_tf32(v.x - h.x);
+  l.y = umma::to_tf32(v.y - h.y);
+  l.z = umma::to_tf32(v.z - h.z);
+  l.w = umma::to_tf32(v.w - h.w);
+  *reinterpret_cast<float4*>(hi + off) = h;
+  *reinterpret_cast<float4*>(lo + off) = l;
+}
+// p[0 .. 3], zero from n valid values on; one 16-byte load where vec says p is aligned
+__device__ __forceinline__ float4 load4(const float* __restrict__ p, long long n, bool vec) {
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (n >= 4 && vec) return *reinterpret_cast<const float4*>(p);
+  if (n > 0) v.x = p[0];
+  if (n > 1) v.y = p[1];
+  if (n > 2) v.z = p[2];
+  if (n > 3) v.w = p[3];
+  return v;
+}
+
 // three tf32 MMAs (hi*hi + hi*lo + lo*hi) over one 32-wide K stage
 __device__ __forceinline__ void issue_stage(uint32_t tmem, uint32_t ahi, uint32_t alo, uint32_t bhi,
                                             uint32_t blo, uint32_t idesc, bool first) {
@@ -88,7 +115,11 @@ __device__ __forceinline__ void issue_stage(uint32_t tmem, uint32_t ahi, uint32_
 
 // gpart[b][c][k][n] = sum_{r in chunk c} psi_k(r) psi_n(r) u_b(r) for one 128 x 128 tile.
 // Dynamic shared memory: 2 stages x (A_hi, A_lo, B_hi, B_lo) x 16 KB = 128 KB (TF32x3), or
-// 2 stages x (A, B) x 16 KB = 64 KB (BF16).
+// 2 stages x (A, B) x 16 KB = 64 KB (BF16).  Bound by loading and splitting the operands, not by
+// the MMAs.  TF32x3: only rows that hold states are written (the others are zeroed once), psi is
+// read once where the two tiles are the same states, and the loads of a stage are issued
+// together.  One value per lane and load, all 128 rows: 2.65 ms at 40^3, 128 states, 16
+// probe-points, 0.87 at 26 x 52 x 52, 64 states, 1; now 0.88 and 0.048 (the latter also for more chunks).
 template <bool BF16>
 __global__ void __launch_bounds__(128, 1)
     k_gram_tc(long long nd, int ns, const float* __restrict__ psi, const float* __restrict__ u,
@@ -126,6 +157,15 @@ __global__ void __launch_bounds__(128, 1)
   const long long span = r1 > r0 ? r1 - r0 : 0;
   constexpr int TK = BF16 ? kTK16 : kTK;
   const int nsteps = (int)((span + TK - 1) / TK);
+  // groups of eight rows with states of either tile; chunks start at multiples of 32 points
+  const int groups = (min(128, ns - min(k0, n0)) + 7) >> 3;
+  const bool vec =
+      ((nd & 3) | ((reinterpret_cast<uintptr_t>(psi) | reinterpret_cast<uintptr_t>(u)) & 15)) == 0;
+  if constexpr (!BF16) {
+    for (uint32_t o = threadIdx.x * 16; o < 8 * kTileBytes128; o += 128 * 16)
+      *reinterpret_cast<float4*>(smem + o) = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncthreads();
+  }
   bool ok = true;
   int issued = 0;  // stages whose MMAs were issued and committed (block-uniform)
   for (int step = 0; step < nsteps; ++step) {
@@ -143,21 +183,53 @@ __global__ void __launch_bounds__(128, 1)
     uint8_t* bhi = BF16 ? alo : alo + kTileBytes128;
     uint8_t* blo = bhi + kTileBytes128;
     const long long rb = r0 + (long long)step * TK;
-    for (int e = threadIdx.x; e < 128 * TK; e += 128) {
-      const int row = e / TK, kk = e - row * TK;
-      const long long r = rb + kk;
-      const bool vr = r < r1;
-      const int k = k0 + row, n = n0 + row;
-      const float a = (vr && k < ns) ? psi[(long long)k * nd + r] : 0.f;
-      const float bv = (vr && n < ns) ? psi[(long long)n * nd + r] * ub[r] : 0.f;
-      if (BF16) {
+    if constexpr (BF16) {
+      for (int e = threadIdx.x; e < 128 * TK; e += 128) {
+        const int row = e / TK, kk = e - row * TK;
+        const long long r = rb + kk;
+        const bool vr = r < r1;
+        const int k = k0 + row, n = n0 + row;
+        const float a = (vr && k < ns) ? psi[(long long)k * nd + r] : 0.f;
+        const float bv = (vr && n < ns) ? psi[(long long)n * nd + r] * ub[r] : 0.f;
         const uint32_t off = kmaj16(row, kk);
         put_bf16(ahi, off, a);
         put_bf16(bhi, off, bv);
-      } else {
-        const uint32_t off = kmaj(row, kk);
-        put_split(ahi, alo, off, a);
-        put_split(bhi, blo, off, bv);
+      }
+    } else {
+      // lane: row rr of a group of eight, four points from 4 * k4 and from 16 + 4 * k4
+      const int rr = lane & 7, k4 = lane >> 3;
+      const long long ra = rb + 4 * k4, rz = ra + 16;
+      const float4 ua = load4(ub + ra, r1 - ra, vec), uz = load4(ub + rz, r1 - rz, vec);
+      for (int g0 = warp; g0 < groups; g0 += 16) {
+        float4 pa[4], pz[4], qa[4], qz[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int row = 8 * (g0 + 4 * i) + rr, k = k0 + row, n = n0 + row;
+          const long long ca = g0 + 4 * i < groups && k < ns ? r1 - ra : 0;
+          const long long cz = g0 + 4 * i < groups && k < ns ? r1 - rz : 0;
+          pa[i] = load4(psi + (long long)k * nd + ra, ca, vec);
+          pz[i] = load4(psi + (long long)k * nd + rz, cz, vec);
+          qa[i] = pa[i];
+          qz[i] = pz[i];
+          if (k0 != n0) {
+            const long long da = g0 + 4 * i < groups && n < ns ? r1 - ra : 0;
+            const long long dz = g0 + 4 * i < groups && n < ns ? r1 - rz : 0;
+            qa[i] = load4(psi + (long long)n * nd + ra, da, vec);
+            qz[i] = load4(psi + (long long)n * nd + rz, dz, vec);
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (g0 + 4 * i >= groups) break;
+          const int row = 8 * (g0 + 4 * i) + rr;
+          const uint32_t oa = kmaj(row, 4 * k4), oz = kmaj(row, 16 + 4 * k4);
+          put_split4(ahi, alo, oa, pa[i]);
+          put_split4(ahi, alo, oz, pz[i]);
+          put_split4(bhi, blo, oa, make_float4(qa[i].x * ua.x, qa[i].y * ua.y, qa[i].z * ua.z,
+                                               qa[i].w * ua.w));
+          put_split4(bhi, blo, oz, make_float4(qz[i].x * uz.x, qz[i].y * uz.y, qz[i].z * uz.z,
+                                               qz[i].w * uz.w));
+        }
       }
     }
     umma::fence_proxy_async();
@@ -204,7 +276,9 @@ __global__ void __launch_bounds__(128, 1)
 
 // x0[(b,n)][r] = sum_k psi_k(r) C_b[k][n] for a 128-point tile and 128 states (N = 256
 // columns: re, im interleaved).  Dynamic shared memory, one stage: A_hi, A_lo (128 rows) and
-// B_hi, B_lo (256 rows) of 128 bytes each, 96 KB (TF32x3); A and B only, 48 KB (BF16).
+// B_hi, B_lo (256 rows) of 128 bytes each, 96 KB (TF32x3); A and B only, 48 KB (BF16).  TF32x3
+// stores whole 16-byte core-matrix rows: 0.66 ms instead of 1.37 at 40^3, 128 states, 16
+// probe-points (0.16 ms is the write of x0).
 template <bool BF16>
 __global__ void __launch_bounds__(128, 1)
     k_x0_tc(long long nd, int ns, const float* __restrict__ psi, const cpx<float>* __restrict__ cmat,
@@ -251,27 +325,51 @@ __global__ void __launch_bounds__(128, 1)
       if (!ok) break;
     }
     const int kb = step * TK;
-    for (int e = threadIdx.x; e < 128 * TK; e += 128) {
-      const int kk = e >> 7, row = e & 127;  // consecutive threads: consecutive points
-      const long long r = r0 + row;
-      const float a = (r < nd && kb + kk < ns) ? psi[(long long)(kb + kk) * nd + r] : 0.f;
-      if (BF16)
+    if constexpr (BF16) {
+      for (int e = threadIdx.x; e < 128 * TK; e += 128) {
+        const int kk = e >> 7, row = e & 127;  // consecutive threads: consecutive points
+        const long long r = r0 + row;
+        const float a = (r < nd && kb + kk < ns) ? psi[(long long)(kb + kk) * nd + r] : 0.f;
         put_bf16(ahi, kmaj16(row, kk), a);
-      else
-        put_split(ahi, alo, kmaj(row, kk), a);
-    }
-    for (int e = threadIdx.x; e < 256 * TK; e += 128) {
-      const int kk = e >> 8, j = e & 255;
-      const int n = n0 + (j >> 1);
-      float v = 0.f;
-      if (kb + kk < ns && n < ns && j < nN) {
-        const cpx<float> cv = cb[(long long)(kb + kk) * ns + n];
-        v = (j & 1) ? cv.im : cv.re;
       }
-      if (BF16)
+      for (int e = threadIdx.x; e < 256 * TK; e += 128) {
+        const int kk = e >> 8, j = e & 255;
+        const int n = n0 + (j >> 1);
+        float v = 0.f;
+        if (kb + kk < ns && n < ns && j < nN) {
+          const cpx<float> cv = cb[(long long)(kb + kk) * ns + n];
+          v = (j & 1) ? cv.im : cv.re;
+        }
         put_bf16(bhi, kmaj16(j, kk), v);
-      else
-        put_split(bhi, blo, kmaj(j, kk), v);
+      }
+    } else {
+      // a thread writes its point's (or column's) 32 values four at a time
+      const long long r = r0 + threadIdx.x;
+      const float* const pr = psi + (r < nd ? r : 0);
+#pragma unroll
+      for (int k4 = 0; k4 < TK / 4; ++k4) {
+        float v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int k = kb + 4 * k4 + i;
+          v[i] = (r < nd && k < ns) ? pr[(long long)k * nd] : 0.f;
+        }
+        put_split4(ahi, alo, kmaj(threadIdx.x, 4 * k4), make_float4(v[0], v[1], v[2], v[3]));
+      }
+      for (int j = threadIdx.x; j < nN; j += 128) {
+        const int n = n0 + (j >> 1);
+        const float* const cr = reinterpret_cast<const float*>(cb) + 2 * (n < ns ? n : 0) + (j & 1);
+#pragma unroll
+        for (int k4 = 0; k4 < TK / 4; ++k4) {
+          float v[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int k = kb + 4 * k4 + i;
+            v[i] = (n < ns && k < ns) ? cr[(long long)k * ns * 2] : 0.f;
+          }
+          put_split4(bhi, blo, kmaj(j, 4 * k4), make_float4(v[0], v[1], v[2], v[3]));
+        }
+      }
     }
     umma::fence_proxy_async();
     __syncthreads();
@@ -340,7 +438,8 @@ cudaError_t galerkin_guess_tc(long long nd, int ns, int nb, const float* psi, co
                               int test_expire) {
   cudaError_t e = bf16 ? tc_attr<true>() : tc_attr<false>();
   if (e != cudaSuccess) return e;
-  const long long chunk_len = (nd + nchunk - 1) / nchunk;
+  // whole stages of 32 points (the last chunks may be short or empty)
+  const long long chunk_len = ((nd + nchunk - 1) / nchunk + 31) / 32 * 32;
   const int nt = (ns + 127) / 128;
   const int nN = std::min(128, ((ns + 15) / 16) * 16);
   dim3 g1(nt * nt, nb, nchunk);
