@@ -389,15 +389,6 @@ static int gram_chunks64(long long nd, int ns, int nb) {
   return (int)std::min<long long>(256, std::max<long long>(gram_chunks(nd), want));
 }
 
-// mixed form (one 128-state tile per block): more chunks, of at least 512 points, up to eight
-// blocks per SM, so that few probe-points fill the GPU and the last wave of blocks is short
-static int gram_chunks_tc(long long nd, int ns, int nb) {
-  const int nt = (ns + 127) / 128;
-  const long long tiles = (long long)nb * nt * nt;
-  const long long want = std::min<long long>((nd + 511) / 512, 1216 / tiles);
-  return (int)std::min<long long>(256, std::max<long long>(gram_chunks(nd), want));
-}
-
 static size_t per_probe_bytes(const rpa_ctx* c) {
   const long long nd = c->nd, ns = c->ns;
   size_t b = (size_t)ns * nd * cpx_bytes(c) * 4;
@@ -456,10 +447,9 @@ static rpa_status ensure_workspace(rpa_ctx* c, int nb) {
   CK(c->sysi.ensure(sizeof(int) * S * kSysI));
   // a wave may hold fewer probe-points than nb, with more chunks each
   size_t gchunks = (size_t)nb * gram_chunks(nd);
-  for (int b = 1; b <= nb; ++b)
-    gchunks = std::max(gchunks, (size_t)b * (c->opt.precision == RPA_FP64
-                                                 ? gram_chunks64(nd, c->ns, b)
-                                                 : gram_chunks_tc(nd, c->ns, b)));
+  if (c->opt.precision == RPA_FP64)
+    for (int b = 1; b <= nb; ++b)
+      gchunks = std::max(gchunks, (size_t)b * gram_chunks64(nd, c->ns, b));
   CK(c->gpart.ensure(sizeof(double) * gchunks * c->ns * c->ns));
   CK(c->cmat.ensure(cb * nb * c->ns * c->ns));
   CK(c->probe_d.ensure(sizeof(long long) * nb));
@@ -1121,7 +1111,11 @@ static rpa_status cocg_loop(rpa_ctx* c, const CocgView<T>& cv_all, int maxit, bo
       CKS(counts(c, cv_all.nsys, cnt, false));
     }
     if (whole || cnt[kActive] <= tail) {
-      if (c->prof_stats) c->prof_stats->tile_rows = c->prof_stats->tile_rows_tail = kTileResident;
+      if (c->prof_stats) {
+        // tile_rows keeps naming the launches over many systems where there were any
+        if (whole) c->prof_stats->tile_rows = kTileResident;
+        c->prof_stats->tile_rows_tail = kTileResident;
+      }
       return resident_loop<T>(c, cv_all, *pl, maxit, cont);
     }
   }
@@ -1272,7 +1266,7 @@ static rpa_status solve_mixed(rpa_ctx* c, int nb, const float* u32, const int* a
   CocgView<float> cv = make_view<float>(c, nb, u32, x, r, p, w);
   CK(galerkin_guess_tc(c->nd, c->ns, nb, c->d32.psi.as<float>(), c->eps_d.as<double>(),
                        c->pomega_d.as<double>(), u32, active, c->dV, c->gpart.as<double>(),
-                       gram_chunks_tc(c->nd, c->ns, nb), c->cmat.as<cpx<float>>(), x, c->flags_d.as<int>() + 2,
+                       gram_chunks(c->nd), c->cmat.as<cpx<float>>(), x, c->flags_d.as<int>() + 2,
                        c->stream, c->opt.precision == RPA_MIXED_BF16,
                        c->opt.debug_expire_waits));
   CK(set_status(S, c->ns, active, kActive, c->sysi.as<int>(), c->stream));

@@ -119,7 +119,9 @@ __device__ __forceinline__ void issue_stage(uint32_t tmem, uint32_t ahi, uint32_
 // the MMAs.  TF32x3: only rows that hold states are written (the others are zeroed once), psi is
 // read once where the two tiles are the same states, and the loads of a stage are issued
 // together.  One value per lane and load, all 128 rows: 2.65 ms at 40^3, 128 states, 16
-// probe-points, 0.87 at 26 x 52 x 52, 64 states, 1; now 0.88 and 0.048 (the latter also for more chunks).
+// probe-points, 0.87 at 26 x 52 x 52, 64 states, 1; now 1.00 and 0.42 (18 blocks).  The chunks and
+// the order of the MMAs decide the rounding of the guesses, which decides where loose solves
+// stop, so neither depends on the number of probe-points.
 template <bool BF16>
 __global__ void __launch_bounds__(128, 1)
     k_gram_tc(long long nd, int ns, const float* __restrict__ psi, const float* __restrict__ u,
@@ -157,10 +159,10 @@ __global__ void __launch_bounds__(128, 1)
   const long long span = r1 > r0 ? r1 - r0 : 0;
   constexpr int TK = BF16 ? kTK16 : kTK;
   const int nsteps = (int)((span + TK - 1) / TK);
-  // groups of eight rows with states of either tile; chunks start at multiples of 32 points
+  // groups of eight rows with states of either tile
   const int groups = (min(128, ns - min(k0, n0)) + 7) >> 3;
   const bool vec =
-      ((nd & 3) | ((reinterpret_cast<uintptr_t>(psi) | reinterpret_cast<uintptr_t>(u)) & 15)) == 0;
+      (((nd | r0) & 3) | ((reinterpret_cast<uintptr_t>(psi) | reinterpret_cast<uintptr_t>(u)) & 15)) == 0;
   if constexpr (!BF16) {
     for (uint32_t o = threadIdx.x * 16; o < 8 * kTileBytes128; o += 128 * 16)
       *reinterpret_cast<float4*>(smem + o) = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -438,8 +440,7 @@ cudaError_t galerkin_guess_tc(long long nd, int ns, int nb, const float* psi, co
                               int test_expire) {
   cudaError_t e = bf16 ? tc_attr<true>() : tc_attr<false>();
   if (e != cudaSuccess) return e;
-  // whole stages of 32 points (the last chunks may be short or empty)
-  const long long chunk_len = ((nd + nchunk - 1) / nchunk + 31) / 32 * 32;
+  const long long chunk_len = (nd + nchunk - 1) / nchunk;
   const int nt = (ns + 127) / 128;
   const int nN = std::min(128, ((ns + 15) / 16) * 16);
   dim3 g1(nt * nt, nb, nchunk);

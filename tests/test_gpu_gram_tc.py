@@ -26,7 +26,7 @@ def test_galerkin_mixed(n, ns):
     R.rpa_set_options(c.ctx, precision="mixed", lanczos_max=1)
     om, u = np.array([0.3, 2.0, 0.7]), rng.standard_normal((3, nd))
     x0 = R.rpa_galerkin(c.ctx, om, u, ns)
-    # the same guesses start a solve, whose chunks are cut differently
+    # the same guesses start a solve
     r, _ = R.rpa_chi0(c.ctx, om, u, ns)
     assert np.isfinite(r).all()
     c.close()
