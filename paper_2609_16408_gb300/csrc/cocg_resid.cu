@@ -330,13 +330,36 @@ Tile tile_of(int nx, int ny, int nz_chunks, int max_tiles, size_t value) {
   return best;
 }
 
+// Planes per block: fewer where the blocks do not fill the GPU, or fill it by a little more than
+// whole waves.  A block loads 2R planes ahead of its first one, about the time of four.
+// FP64, 8 systems on 12^3 (8 blocks): 67 -> 11 us; double-float, 64 systems on 26 x 52 x 52 (384
+// blocks of which 304 run at once): 452 -> 361 us.
+// Two-die GB300: 152 SMs; a wrong count costs time only.
+constexpr int kSMs = 152;
+int z_chunk(int nz, int zchunk, long long blocks, int max_chunks, int slots) {
+  int best = zchunk;
+  long long best_cost = 0;
+  for (int c = (nz + zchunk - 1) / zchunk; c <= std::min(max_chunks, nz); ++c) {
+    const int len = (nz + c - 1) / c, n = (nz + len - 1) / len;
+    const long long cost = (blocks * n + slots - 1) / slots * (len + 4);
+    if (best_cost == 0 || cost < best_cost) {
+      best_cost = cost;
+      best = len;
+    }
+  }
+  return best;
+}
+
 template <typename T, typename TL, int R>
 void launch_r(const CocgView<T>& cv, const cpx<T>* x, cpx<T>* r, cpx<T>* pdir, int mask,
               cpx<TL>* r_lo, cpx<TL>* p_lo, cpx<TL>* x_lo, bool use_df,
               const cpx<TL>* p_keep, const DfAux& aux, cudaStream_t s) {
   const int nx = cv.st.nx, ny = cv.st.ny, nz = cv.st.nz;
-  const int zchunk = nz <= 64 ? nz : 32, nzc = (nz + zchunk - 1) / zchunk;
+  int zchunk = nz <= 64 ? nz : 32, nzc = (nz + zchunk - 1) / zchunk;
   const Tile t = tile_of<R>(nx, ny, nzc, cv.tiles, sizeof(cpx<T>));
+  zchunk = z_chunk(nz, zchunk, (long long)t.n * cv.nsys, cv.tiles / t.n,
+                   kSMs * (sizeof(T) == 4 ? 3 : 2) * (kRThreads / ((t.tx * t.ty + 31) / 32 * 32)));
+  nzc = (nz + zchunk - 1) / zchunk;
   const size_t planes = 2 * sizeof(cpx<T>) * (t.tx + 2 * R) * (t.ty + 2 * R);
   size_t cdb = sizeof(cpx<T>) * cv.nl.ngroup * kProjChunk;
   if (cdb + planes + 1024 > 48 * 1024) cdb = 0;
