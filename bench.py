@@ -337,6 +337,8 @@ def run_ours(args, wl):
         if t <= -101:
             return (f"bands of {-100 - t} full x rows, two x points per thread, 3-stage "
                     "cp.async pipeline")
+        if t == -7:
+            return "whole COCG loop in one kernel, a cluster per system"
         if t == -6:
             return "two-point kernel on packed full rows"
         if t in (-3, -4):
@@ -347,6 +349,7 @@ def run_ours(args, wl):
     hname = ("k_dirmatvec_band" if tile_rows <= -101
              else "k_dirmatvec_rows" if tile_rows > 0
              else "k_dirmatvec_x2p" if tile_rows == -6
+             else "k_cocg_resident" if tile_rows == -7
              else ("k_dirmatvec_x2" if tile_rows in (-2, -3, -4) else "k_dirmatvec"))
     names = ["proj_dots", hname, "k_scalars", "k_update_dots", "none"]
     dom = 1 if ks[1] >= ks[3] else 3
@@ -365,7 +368,11 @@ def run_ours(args, wl):
             # per-system bytes of the captured grid, scaled to this grid's point count
             scale = nd / tj.get("grid_points", nd)
             traffic = tj["dram_bytes_per_system"] * scale * sys_per_launch
-    roofline = dict(bound="hbm", kernel=names[dom], achieved=achieved, peak=pk["hbm_gbs"],
+    both = dom == 1 and tile_tail == -7 and tile_rows != -7
+    if both:  # launches of two kernels in one class: no per-launch traffic
+        traffic = None
+    roofline = dict(bound="hbm", kernel=names[dom] + (" + k_cocg_resident" if both else ""),
+                    achieved=achieved, peak=pk["hbm_gbs"],
                     unit="GB/s", frac=achieved / pk["hbm_gbs"], traffic=traffic,
                     algorithmic_bytes_per_launch=float(kb[dom] / max(1, kl[dom])),
                     peak_src=pk["src"] + " (burst copy)",
@@ -643,7 +650,8 @@ def run_interp_sweep(args, wl):
 
 _KERNEL_FILES = {"k_dirmatvec": "cocg_fused.cu", "k_update_dots": "cocg_fused.cu",
                  "k_dirmatvec_x2": "cocg_x2.cu", "k_dirmatvec_rows": "cocg_rows.cu",
-                 "k_dirmatvec_band": "cocg_band.cu", "k_dirmatvec_x2p": "cocg_x2p.cu"}
+                 "k_dirmatvec_band": "cocg_band.cu", "k_dirmatvec_x2p": "cocg_x2p.cu",
+                 "k_cocg_resident": "cocg_resident.cu"}
 
 
 def kernel_source_sha(kernel="k_dirmatvec"):

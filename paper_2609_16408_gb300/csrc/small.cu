@@ -224,7 +224,7 @@ __global__ void k_ec_partial(long long nd, int nw, const double* __restrict__ df
 }
 
 // One block: 256 strided sums in order, then a tree (a single thread took 71 us for 1,370
-// partial sums, one FP64 addition of 64 cycles after the other; 4 us now).
+// partial sums, one FP64 addition of 64 cycles after the other; 2.9 us now).
 __global__ void __launch_bounds__(256) k_ec_final(int n, const double* __restrict__ part,
                                                   double* __restrict__ ec) {
   double t = 0.0;
@@ -274,8 +274,8 @@ cudaError_t interp_taps(int n, int m, const double* Wt, int4* ti, double* tw, cu
 
 // Interpolation along one axis by the taps: out[i2][a][i0] = sum_t w_t(a) in[i2][ti_t(a)][i0],
 // i0 < inner, a < nout, and with part the block's sum of the outputs times weight[b].  Bound by
-// the FP64 pipe (4 multiply-adds per output of the last axis, 19 us for ten 52^3 arrays); the
-// dense mode product did one per coarse node, 26 of them, nearly all with weight 0: 125 us.
+// the FP64 pipe (4 multiply-adds per output): 36 us for the three axes of ten 52^3 arrays; the
+// dense mode products did one per coarse node, 26 of them, nearly all with weight 0: 120 us.
 constexpr int kTapOut = 4;  // outputs per thread
 __global__ void __launch_bounds__(256) k_taps(const double* __restrict__ in, long long in_bs,
                                               double* __restrict__ out, long long out_bs,
