@@ -181,9 +181,10 @@ __device__ __forceinline__ bool acc_le(df a, df b) { return a.hi < b.hi || (a.hi
 // (ar + i ai) / (br + i bi)
 __device__ __forceinline__ void acc_cdiv(double ar, double ai, double br, double bi, double& qr,
                                          double& qi) {
-  const double inv = 1.0 / (br * br + bi * bi);
-  qr = (ar * br + ai * bi) * inv;
-  qi = (ai * br - ar * bi) * inv;
+  // two quotients: the reciprocal of a |b|^2 below 2^-1024 would overflow
+  const double den = br * br + bi * bi;
+  qr = (ar * br + ai * bi) / den;
+  qi = (ai * br - ar * bi) / den;
 }
 __device__ __forceinline__ void acc_cdiv(df ar, df ai, df br, df bi, float& qr, float& qi) {
   // scaled by a power of two near 1 / |b|, so that the products neither overflow nor vanish
