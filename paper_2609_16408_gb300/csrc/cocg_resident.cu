@@ -142,66 +142,26 @@ __device__ __forceinline__ int tid() {
 __device__ __forceinline__ int quot(int a, unsigned magic) { return (int)__umulhi((unsigned)a, magic); }
 
 // ---- per-system scalars ------------------------------------------------------------------
-// The sums over warps and blocks and the quotients alpha and beta are FP64 in the FP64 form.
-// In the FP32 form the terms are FP32 sums and the quotients are rounded to FP32, and they
-// are formed in double-float arithmetic (about 48 bits): FP64 instructions take 64 cycles
-// each on this GPU and the serial chain of one scalar step 4,000.
-template <typename T>
-struct Acc;
-template <>
-struct Acc<double> {
-  using A = double;
-};
-template <>
-struct Acc<float> {
-  using A = df;
-};
-__device__ __forceinline__ double acc_of(double v) { return v; }
-__device__ __forceinline__ df acc_of(float v) { return df{v, 0.f}; }
-__device__ __forceinline__ double acc_add(double a, double b) { return a + b; }
-__device__ __forceinline__ df acc_add(df a, df b) { return df_add(a, b); }
-__device__ __forceinline__ double acc_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
-__device__ __forceinline__ df acc_xor(df v, int o) {
-  return df{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
+// The sums over warps and blocks, rho, ||r||^2, its target and the quotients alpha and beta are
+// FP64 in both forms, as in the launched iteration.  An FP64 instruction takes 64 cycles of a
+// warp whatever its active lanes, so the values that belong together go through one instruction
+// in lanes of their own, and what can be read off the bits is.
+__device__ __forceinline__ bool finite_bits(double v) {
+  return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000;
 }
-__device__ __forceinline__ double acc_lane(double v, int l) { return __shfl_sync(0xffffffffu, v, l); }
-__device__ __forceinline__ df acc_lane(df v, int l) {
-  return df{__shfl_sync(0xffffffffu, v.hi, l), __shfl_sync(0xffffffffu, v.lo, l)};
+__device__ __forceinline__ bool zero_bits(double v) {
+  return ((__double2hiint(v) & 0x7fffffff) | __double2loint(v)) == 0;
 }
-__device__ __forceinline__ double acc_val(double v) { return v; }
-__device__ __forceinline__ double acc_val(df v) { return df_val(v); }
-__device__ __forceinline__ void acc_from(double& a, double v) { a = v; }
-__device__ __forceinline__ void acc_from(df& a, double v) { a = df_of(v); }
-__device__ __forceinline__ bool acc_zero(double v) { return v == 0.0; }
-__device__ __forceinline__ bool acc_zero(df v) { return v.hi == 0.f; }
-__device__ __forceinline__ bool acc_finite(double v) { return isfinite(v); }
-__device__ __forceinline__ bool acc_finite(df v) { return isfinite(v.hi); }
-__device__ __forceinline__ bool acc_le(double a, double b) { return a <= b; }
-__device__ __forceinline__ bool acc_le(df a, df b) { return a.hi < b.hi || (a.hi == b.hi && a.lo <= b.lo); }
-// (ar + i ai) / (br + i bi)
-__device__ __forceinline__ void acc_cdiv(double ar, double ai, double br, double bi, double& qr,
-                                         double& qi) {
-  // two quotients: the reciprocal of a |b|^2 below 2^-1024 would overflow
-  const double den = br * br + bi * bi;
-  qr = (ar * br + ai * bi) / den;
-  qi = (ai * br - ar * bi) / den;
+// a <= b for finite values >= 0
+__device__ __forceinline__ bool le_bits(double a, double b) {
+  return __double_as_longlong(a) <= __double_as_longlong(b);
 }
-__device__ __forceinline__ void acc_cdiv(df ar, df ai, df br, df bi, float& qr, float& qi) {
-  // scaled by a power of two near 1 / |b|, so that the products neither overflow nor vanish
-  const float m = fmaxf(fabsf(br.hi), fabsf(bi.hi));
-  int e = (__float_as_int(m) >> 23) & 0xff;
-  e = min(max(254 - e, 1), 253);
-  const float sc = __int_as_float(e << 23);
-  br = df{br.hi * sc, br.lo * sc};
-  bi = df{bi.hi * sc, bi.lo * sc};
-  ar = df{ar.hi * sc, ar.lo * sc};
-  ai = df{ai.hi * sc, ai.lo * sc};
-  const df den = df_fma(df_mul(br, br), bi, bi);
-  const df nr = df_fma(df_mul(ar, br), ai, bi), ni = df_fma(df_mul(ai, br), df_neg(ar), bi);
-  // one correction from the exact remainder rounds the quotient of the pairs
-  const float q0 = nr.hi / den.hi, q1 = ni.hi / den.hi;
-  qr = q0 + df_fma(nr, df{-q0, 0.f}, den).hi / den.hi;
-  qi = q1 + df_fma(ni, df{-q1, 0.f}, den).hi / den.hi;
+// (ar + i ai) / (br + i bi): the real part in even lanes, the imaginary part in odd ones.  A
+// division, not a product with the reciprocal of |b|^2: that of a subnormal |b|^2 overflows.
+__device__ __forceinline__ double cdiv_lanes(double ar, double ai, double br, double bi, int lane) {
+  const bool im = (lane & 1) != 0;
+  const double p = im ? ai : ar, q = im ? -ar : ai;
+  return (p * br + q * bi) / (br * br + bi * bi);
 }
 
 template <typename T>
@@ -221,16 +181,15 @@ template <typename T>
 struct alignas(16) Brick {
   using V = typename Val<T>::V;
   using K = typename Val<T>::K;
-  using A = typename Acc<T>::A;
   V *xg, *rg, *pg;  // x, r and p of the system in global memory
   int nx, ny, nz, y0, z0, by, bz, pitch, cap, nslot, rank, ng4;
   int px, py, pz;  // periodic axes
   T eps, om, be_r, be_i, al_r, al_i;
-  A rho_r, rho_i, rn2, target2;
+  double rho_r, rho_i, rn2, target2;
   int ctl, iters;
   K kc[3 * (kMaxRadius + 1)];  // stencil coefficients per axis
   T red[32 * 4];
-  A slots2[kResMaxCluster * 4], slots3[kResMaxCluster * 4];
+  double slots2[kResMaxCluster * 4], slots3[kResMaxCluster * 4];
   Args<T> a;  // the launch's arguments
   // offsets of the vectors: p at 0, w, r and x (if resident), projector sums and coefficients
   __device__ int off_w() const { return cap; }
@@ -537,7 +496,7 @@ __device__ __noinline__ cpx<T> part_y() {
 // Sums of NQ (2 or 4) values over the block; every lane of warp 0 gets them.  Within a warp the
 // lanes exchange halves of the values first, so that each adds one value in the end.
 template <typename T, int NQ>
-__device__ __forceinline__ void block_total(T (&v)[NQ], T* red, typename Acc<T>::A (&out)[NQ]) {
+__device__ __forceinline__ void block_total(T (&v)[NQ], T* red, double (&out)[NQ]) {
   const int lane = tid() & 31, wid = tid() >> 5, nw = blockDim.x >> 5;
   int o = 16, q = 0;
 #pragma unroll
@@ -558,37 +517,37 @@ __device__ __forceinline__ void block_total(T (&v)[NQ], T* red, typename Acc<T>:
     // one tree for all values together (FP64 additions take 64 cycles of the pipe each)
     constexpr int S = 32 / NQ;
     const int qq = lane / S, w = lane % S;
-    typename Acc<T>::A t = acc_of(w < nw ? red[w * NQ + qq] : (T)0);
-    if (nw > S) t = acc_add(t, acc_of(w + S < nw ? red[(w + S) * NQ + qq] : (T)0));
+    double t = w < nw ? (double)red[w * NQ + qq] : 0.0;
+    if (nw > S) t += w + S < nw ? (double)red[(w + S) * NQ + qq] : 0.0;
 #pragma unroll
-    for (int x = S / 2; x > 0; x >>= 1) t = acc_add(t, acc_xor(t, x));
+    for (int x = S / 2; x > 0; x >>= 1)
+      if (x < nw) t += __shfl_xor_sync(0xffffffffu, t, x);
 #pragma unroll
-    for (int i = 0; i < NQ; ++i) out[i] = acc_lane(t, i * S);
+    for (int i = 0; i < NQ; ++i) out[i] = __shfl_sync(0xffffffffu, t, i * S);
   }
 }
 
 // Sum over the blocks of the cluster: warp 0 puts the block's totals into every block's slots;
 // after the barrier warp 0 of each block adds the slots in a fixed tree.
-template <typename A, int NQ>
-__device__ __forceinline__ void post_totals(cg::cluster_group& cl, const A (&v)[NQ], A* slots,
-                                            int G, int rank) {
+template <int NQ>
+__device__ __forceinline__ void post_totals(cg::cluster_group& cl, const double (&v)[NQ],
+                                            double* slots, int G, int rank) {
   if ((int)threadIdx.x < G) {
-    A* dst = cl.map_shared_rank(slots, threadIdx.x);
+    double* dst = cl.map_shared_rank(slots, threadIdx.x);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) dst[rank * 4 + q] = v[q];
   }
 }
-template <typename T, int NQ>
-__device__ __forceinline__ void read_totals(const typename Acc<T>::A* slots, int G,
-                                            typename Acc<T>::A (&v)[NQ]) {
+template <int NQ>
+__device__ __forceinline__ void read_totals(const double* slots, int G, double (&v)[NQ]) {
   // value q of blocks r, r + 32 / NQ in lane q * (32 / NQ) + r
   constexpr int S = 32 / NQ;
   const int lane = threadIdx.x & 31, q = lane / S, r = lane % S;
-  typename Acc<T>::A t = r < G ? slots[r * 4 + q] : acc_of((T)0);
-  if (G > S) t = acc_add(t, r + S < G ? slots[(r + S) * 4 + q] : acc_of((T)0));
-  for (int x = 1; x < G && x < S; x <<= 1) t = acc_add(t, acc_xor(t, x));
+  double t = r < G ? slots[r * 4 + q] : 0.0;
+  if (G > S) t += r + S < G ? slots[(r + S) * 4 + q] : 0.0;
+  for (int x = 1; x < G && x < S; x <<= 1) t += __shfl_xor_sync(0xffffffffu, t, x);
 #pragma unroll
-  for (int i = 0; i < NQ; ++i) v[i] = acc_lane(t, i * S);
+  for (int i = 0; i < NQ; ++i) v[i] = __shfl_sync(0xffffffffu, t, i * S);
 }
 
 #define RES_BY_LEN(l, call) \
@@ -877,7 +836,6 @@ __device__ __noinline__ Sum3<T> phase_update() {
 template <typename T, int R>
 __global__ void __launch_bounds__(max_threads<T>(), 1) k_cocg_resident(const __grid_constant__ Args<T> arg) {
   using V = typename Val<T>::V;
-  using A = typename Acc<T>::A;
   cg::cluster_group cl = cg::this_cluster();
   Brick<T>& k = brick<T>();
   const Args<T>& a = k.a;
@@ -923,10 +881,10 @@ __global__ void __launch_bounds__(max_threads<T>(), 1) k_cocg_resident(const __g
       k.om = (T)a.omega[b];
       k.be_r = a.cont ? (T)sd[kBeta] : (T)0;
       k.be_i = a.cont ? (T)sd[kBeta + 1] : (T)0;
-      acc_from(k.rho_r, sd[kRho]);
-      acc_from(k.rho_i, sd[kRho + 1]);
-      acc_from(k.rn2, sd[kRnorm] * sd[kRnorm]);
-      acc_from(k.target2, sd[kTarget] * sd[kTarget]);
+      k.rho_r = sd[kRho];
+      k.rho_i = sd[kRho + 1];
+      k.rn2 = sd[kRnorm] * sd[kRnorm];
+      k.target2 = sd[kTarget] * sd[kTarget];
       k.iters = a.sysi[(long long)s * kSysI + kIters];
       k.ctl = kActive;
     }
@@ -993,22 +951,24 @@ __global__ void __launch_bounds__(max_threads<T>(), 1) k_cocg_resident(const __g
 #define RES_Y(L) pw = part_y<T, L, R>()
       RES_BY_LEN(a.ly, RES_Y)
       T sum2[2] = {pw.re, pw.im};
-      A tot2[2];
+      double tot2[2];
       block_total<T, 2>(sum2, k.red, tot2);
-      if (tid() < 32) post_totals<A, 2>(cl, tot2, k.slots2, a.G, k.rank);
+      if (tid() < 32) post_totals<2>(cl, tot2, k.slots2, a.G, k.rank);
     }
     cl.sync();
     // alpha = rho / (p^T A p)
     if (tid() < 32) {
-      A tot2[2];
-      read_totals<T, 2>(k.slots2, a.G, tot2);
+      double tot2[2];
+      read_totals<2>(k.slots2, a.G, tot2);
+      const double q = cdiv_lanes(k.rho_r, k.rho_i, tot2[0], tot2[1], tid());
+      if (tid() == 1) k.al_i = (T)q;
       if (tid() == 0) {
+        k.al_r = (T)q;
         if (k.iters >= a.maxit)
           k.ctl = kMaxit;
-        else if ((acc_zero(tot2[0]) && acc_zero(tot2[1])) || !acc_finite(tot2[0]) || !acc_finite(tot2[1]))
+        else if ((zero_bits(tot2[0]) && zero_bits(tot2[1])) || !finite_bits(tot2[0]) ||
+                 !finite_bits(tot2[1]))
           k.ctl = kBreakdown;
-        else
-          acc_cdiv(k.rho_r, k.rho_i, tot2[0], tot2[1], k.al_r, k.al_i);
       }
     }
     __syncthreads();
@@ -1018,23 +978,26 @@ __global__ void __launch_bounds__(max_threads<T>(), 1) k_cocg_resident(const __g
                                  : (a.r_res ? phase_update<T, true, false>()
                                             : phase_update<T, false, false>());
       T sum3[4] = {rr.v[0], rr.v[1], rr.v[2], (T)0};
-      A tot3[4];
+      double tot3[4];
       block_total<T, 4>(sum3, k.red, tot3);
-      if (tid() < 32) post_totals<A, 4>(cl, tot3, k.slots3, a.G, k.rank);
+      if (tid() < 32) post_totals<4>(cl, tot3, k.slots3, a.G, k.rank);
     }
     cl.sync();
     if (tid() < 32) {
-      A tot3[4];
-      read_totals<T, 4>(k.slots3, a.G, tot3);
+      double tot3[4];
+      read_totals<4>(k.slots3, a.G, tot3);
+      const double q = cdiv_lanes(tot3[1], tot3[2], k.rho_r, k.rho_i, tid());
+      __syncwarp();  // every lane has read rho
+      if (tid() == 1) k.be_i = (T)q;
       if (tid() == 0) {
+        k.be_r = (T)q;
         k.iters += 1;
         k.rn2 = tot3[0];
-        if (!acc_finite(tot3[0])) {
+        if (!finite_bits(tot3[0])) {
           k.ctl = kBreakdown;
-        } else if (acc_le(tot3[0], k.target2)) {
-          k.ctl = kConverged;
+        } else if (le_bits(tot3[0], k.target2)) {
+          k.ctl = kConverged;  // rho stays that of the residual of the last direction
         } else {
-          acc_cdiv(tot3[1], tot3[2], k.rho_r, k.rho_i, k.be_r, k.be_i);
           k.rho_r = tot3[1];
           k.rho_i = tot3[2];
         }
@@ -1070,9 +1033,9 @@ __global__ void __launch_bounds__(max_threads<T>(), 1) k_cocg_resident(const __g
     const long long s = (long long)(ci % a.nb) * a.ns + (a.ns - 1 - ci / a.nb);
     double* sd = a.sysd + s * kSysD;
     int* si = a.sysi + s * kSysI;
-    sd[kRho] = acc_val(k.rho_r);
-    sd[kRho + 1] = acc_val(k.rho_i);
-    sd[kRnorm] = sqrt(acc_val(k.rn2));
+    sd[kRho] = k.rho_r;
+    sd[kRho + 1] = k.rho_i;
+    sd[kRnorm] = sqrt(k.rn2);
     si[kIters] = k.iters;
     si[kStatus] = k.ctl;
   }
