@@ -33,6 +33,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <type_traits>
 
 #include "cocg.cuh"
 #include "cocg_resident.cuh"
@@ -188,7 +189,7 @@ struct alignas(16) Brick {
   double rho_r, rho_i, rn2, target2;
   int ctl, iters;
   K kc[3 * (kMaxRadius + 1)];  // stencil coefficients per axis
-  T red[32 * 4];
+  dacc_t<T> red[32 * 4];
   double slots2[kResMaxCluster * 4], slots3[kResMaxCluster * 4];
   Args<T> a;  // the launch's arguments
   // offsets of the vectors: p at 0, w, r and x (if resident), projector sums and coefficients
@@ -429,9 +430,10 @@ __device__ __noinline__ void part_z() {
 
 // y part, diagonal and the end of w: W += y sums + (c0 + V - sigma) p; sums p^T w
 template <typename T, int L, int R>
-__device__ __noinline__ cpx<T> part_y() {
+__device__ __noinline__ cpx<dacc_t<T>> part_y() {
   const Brick<T>& k = brick<T>();
   using V = typename Val<T>::V;
+  using D = dacc_t<T>;
   typename Val<T>::K c[R + 1];
 #pragma unroll
   for (int m = 1; m <= R; ++m) c[m] = k.kc[kMaxRadius + 1 + m];
@@ -447,6 +449,7 @@ __device__ __noinline__ cpx<T> part_y() {
   const T* const vloc = k.a.vloc + plane * k.z0 + nx * k.y0;
   const T c0 = k.a.st.c0, eps = k.eps, om = k.om;
   V sum = vzero<T>();
+  D dre = 0, dim = 0;  // the sum where its type is not T (RPA_DOT_F64)
   const int lane = tid() & 31, nw = blockDim.x >> 5;
 #pragma unroll 1
   for (int u = warp_id(); u < units; u += nw) {
@@ -485,12 +488,20 @@ __device__ __noinline__ cpx<T> part_y() {
         w[i * pitch] = wv;
         T pr, pi;
         parts(pc, pr, pi);
-        sum = cfma(sum, pr, pi, wv);
+        if constexpr (std::is_same<D, T>::value) {
+          sum = cfma(sum, pr, pi, wv);
+        } else {
+          T wr, wi;
+          parts(wv, wr, wi);
+          dre += (D)pr * wr - (D)pi * wi;
+          dim += (D)pr * wi + (D)pi * wr;
+        }
       }
   }
+  if constexpr (!std::is_same<D, T>::value) return mk<D>(dre, dim);
   T sre, sim;
   parts(sum, sre, sim);
-  return mk<T>(sre, sim);
+  return mk<D>(sre, sim);
 }
 
 // Sums of NQ (2 or 4) values over the block; every lane of warp 0 gets them.  Within a warp the
@@ -768,7 +779,7 @@ __device__ __noinline__ void phase_proj_term() {
 // the thread's ||r||^2 and r^T r
 template <typename T>
 struct Sum3 {
-  T v[3];
+  dacc_t<T> v[3];
 };
 // r -= alpha w, x += alpha p; RRES, XRES: r and x in shared memory
 template <typename T, bool RRES, bool XRES>
@@ -783,7 +794,8 @@ __device__ __noinline__ Sum3<T> phase_update() {
            *const xg = k.xg;
   const V *const P = smem_vec<T>(0), *const W = smem_vec<T>(k.off_w());
   const int* const rowoff = k.rowoff();
-  T s0 = 0, s1 = 0, s2 = 0;
+  using D = dacc_t<T>;
+  D s0 = 0, s1 = 0, s2 = 0;
   auto step = [&](int slot, int g, const V& rv, const V& xv, const V& wv, const V& pv) {
     const V r = cfma(rv, -al_r, -al_i, wv), x = cfma(xv, al_r, al_i, pv);
     if (RRES)
@@ -801,9 +813,9 @@ __device__ __noinline__ Sum3<T> phase_update() {
       s1 = fma(im, im, s1);
       s2 = fma(re, im, s2);
     } else {
-      s0 += re * re + im * im;
-      s1 += re * re - im * im;
-      s2 += (T)2 * re * im;
+      s0 += (D)re * re + (D)im * im;
+      s1 += (D)re * re - (D)im * im;
+      s2 += (D)2 * re * im;
     }
   };
   int i0 = tid();
@@ -947,12 +959,12 @@ __global__ void __launch_bounds__(max_threads<T>(), 1) k_cocg_resident(const __g
     __syncthreads();
     if (k.ng4) phase_proj_term<T>();
     {
-      cpx<T> pw;
+      cpx<dacc_t<T>> pw;
 #define RES_Y(L) pw = part_y<T, L, R>()
       RES_BY_LEN(a.ly, RES_Y)
-      T sum2[2] = {pw.re, pw.im};
+      dacc_t<T> sum2[2] = {pw.re, pw.im};
       double tot2[2];
-      block_total<T, 2>(sum2, k.red, tot2);
+      block_total<dacc_t<T>, 2>(sum2, k.red, tot2);
       if (tid() < 32) post_totals<2>(cl, tot2, k.slots2, a.G, k.rank);
     }
     cl.sync();
@@ -977,9 +989,9 @@ __global__ void __launch_bounds__(max_threads<T>(), 1) k_cocg_resident(const __g
       const Sum3<T> rr = a.x_res ? phase_update<T, true, true>()
                                  : (a.r_res ? phase_update<T, true, false>()
                                             : phase_update<T, false, false>());
-      T sum3[4] = {rr.v[0], rr.v[1], rr.v[2], (T)0};
+      dacc_t<T> sum3[4] = {rr.v[0], rr.v[1], rr.v[2], 0};
       double tot3[4];
-      block_total<T, 4>(sum3, k.red, tot3);
+      block_total<dacc_t<T>, 4>(sum3, k.red, tot3);
       if (tid() < 32) post_totals<4>(cl, tot3, k.slots3, a.G, k.rank);
     }
     cl.sync();

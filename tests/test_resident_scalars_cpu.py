@@ -1,6 +1,6 @@
 """Types of the resident COCG kernel's scalars, checked by the compiler: the sums over warps and
 blocks, rho, ||r||^2 and its target are FP64 in the FP32 form too, as in the launched
-iteration."""
+iteration, and with RPA_DOT_F64 = 1 the threads' and warps' dot products are."""
 import os
 import shutil
 import subprocess
@@ -31,3 +31,13 @@ def test_scalars_are_fp64(tmp_path):
         for m in ("rho_r", "rho_i", "rn2", "target2")) + "\n" + "\n".join(
         f"static_assert(same<decltype(Brick<float>::{m}[0]), double>, \"{m}\");"
         for m in ("slots2", "slots3")))
+
+
+@pytest.mark.skipif(shutil.which(NVCC) is None, reason="needs nvcc")
+@pytest.mark.parametrize("flag,want", [("-DRPA_DOT_F64=1", "double"), ("-DRPA_DOT_F64=0", "float")])
+def test_dot_products_follow_the_build_flag(tmp_path, flag, want):
+    compiles(tmp_path, "\n".join(
+        f"static_assert(same<decltype({e}), {want}>, \"{n}\");"
+        for n, e in (("p^T w", "part_y<float, 4, 6>().re"),
+                     ("r^T r", "phase_update<float, true, true>().v[0]"),
+                     ("warp sums", "Brick<float>::red[0]"))), flag)
