@@ -922,7 +922,7 @@ static rpa_status resident_tables(rpa_ctx* c, rpa_ctx::ResidentPlan& pl) {
       const int by = y0[ry[y] + 1] - y0[ry[y]];
       const int slot = ((z - z0[rz[z]]) * by + (y - y0[ry[y]])) * sh.pitch + x;
       const int l = cnt[rank][slot];
-      if (l == 255) {  // more groups at a point than the layers count: the launched iteration
+      if (l == 255) {  // more groups at a point than the layers count
         pl.sh.G = 0;
         return RPA_OK;
       }
@@ -1020,23 +1020,29 @@ static rpa_status resident_plan(rpa_ctx* c, int nsys, rpa_ctx::ResidentPlan** ou
       !resident_supported(c->grid.fd_radius))
     return RPA_OK;
   const int k = sizeof(T) == 4 ? 0 : 1;
-  rpa_ctx::ResidentPlan* best = nullptr;
-  // the fewest blocks whose memory holds p and w: a brick then has the least halo and the
-  // fewest barriers per point; with fewer systems than blocks fit, larger clusters use the rest
-  for (int i = 0; i < 5; ++i) {
-    rpa_ctx::ResidentPlan& pl = c->resident[k][i];
-    if (!pl.known) {
-      CK(resident_shape<T>(c->grid.n[0], c->grid.n[1], c->grid.n[2], c->grid.fd_radius, c->ngroup,
-                           1 << i, &pl.sh));
-      pl.known = true;
+  // a size whose projector tables do not fit drops out (sh.G = 0), and the choice is made again
+  // in the same call, so that it does not depend on the calls before
+  for (;;) {
+    rpa_ctx::ResidentPlan* best = nullptr;
+    // the fewest blocks whose memory holds p and w: a brick then has the least halo and the
+    // fewest barriers per point; with fewer systems than blocks fit, larger clusters use the rest
+    for (int i = 0; i < 5; ++i) {
+      rpa_ctx::ResidentPlan& pl = c->resident[k][i];
+      if (!pl.known) {
+        CK(resident_shape<T>(c->grid.n[0], c->grid.n[1], c->grid.n[2], c->grid.fd_radius,
+                             c->ngroup, 1 << i, &pl.sh));
+        pl.known = true;
+      }
+      if (pl.sh.G == 0) continue;
+      if (!best || nsys <= pl.sh.clusters) best = &pl;
     }
-    if (pl.sh.G == 0) continue;
-    if (!best || nsys <= pl.sh.clusters) best = &pl;
+    if (!best) return RPA_OK;
+    if (!best->tables) CKS(resident_tables<T>(c, *best));
+    if (best->sh.G) {
+      *out = best;
+      return RPA_OK;
+    }
   }
-  if (!best) return RPA_OK;
-  if (!best->tables) CKS(resident_tables<T>(c, *best));
-  if (best->sh.G) *out = best;
-  return RPA_OK;
 }
 
 template <typename T>
