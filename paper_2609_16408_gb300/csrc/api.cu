@@ -1011,11 +1011,26 @@ static rpa_status resident_tables(rpa_ctx* c, rpa_ctx::ResidentPlan& pl) {
 // on (12^3: one probe-point of 20 Lanczos steps in FP64, 144 -> 55 ms).
 constexpr long long kResidentMinPoints = 1536;
 
-// The cluster size for nsys systems, or no plan where the resident kernel does not apply: an
+// The cluster size for n systems, or no plan where the resident kernel does not apply: an
 // explicit tiling or loop mode asks for the launched iteration.
+//
+// The fewest blocks whose memory holds p and w: a brick then has the least halo and the fewest
+// barriers per point.  With few systems larger clusters use the SMs that are left: while at most
+// nine quarters of one cluster per system fit at a time, as systems that end early leave their
+// cluster to the next one.  A size chosen by what fits at a time loses to the launched iteration
+// where 16 systems meet 15 clusters of 8 or 48 meet 36 of 4 (FP64, one vector of 16 states, 26^3:
+// clusters of 4 17.3 ms, launched 15.4, clusters of 8 9.8; 30^3: 27.2 / 20.7 / 15.4; FP32, three
+// vectors, 30^3: clusters of 2 10.2 ms, launched 9.1, clusters of 4 6.6).  At a ratio of 3.2 the
+// larger size was between 27 % ahead and 5 % behind, at 4.3 behind.  FP32 from one block to two:
+// three halves, where the launched iteration may win (23^3, 96 systems: 6.6 against 6.8 ms, two
+// blocks 4.4); with more systems one block is ahead of it and keeps its sums.
+// n: in FP64 the active systems, since most of a wave may be done (26^3, one live vector of 20: 28.8
+// ms by the systems of the wave, 26.4 launched).
 template <typename T>
-static rpa_status resident_plan(rpa_ctx* c, int nsys, rpa_ctx::ResidentPlan** out) {
+static rpa_status resident_plan(rpa_ctx* c, int n, rpa_ctx::ResidentPlan** out,
+                                bool* by_count = nullptr) {
   *out = nullptr;
+  if (by_count) *by_count = false;
   if (c->opt.tile != -1 || c->opt.graphs != 2 || c->nd < kResidentMinPoints ||
       !resident_supported(c->grid.fd_radius))
     return RPA_OK;
@@ -1024,8 +1039,6 @@ static rpa_status resident_plan(rpa_ctx* c, int nsys, rpa_ctx::ResidentPlan** ou
   // in the same call, so that it does not depend on the calls before
   for (;;) {
     rpa_ctx::ResidentPlan* best = nullptr;
-    // the fewest blocks whose memory holds p and w: a brick then has the least halo and the
-    // fewest barriers per point; with fewer systems than blocks fit, larger clusters use the rest
     for (int i = 0; i < 5; ++i) {
       rpa_ctx::ResidentPlan& pl = c->resident[k][i];
       if (!pl.known) {
@@ -1034,9 +1047,14 @@ static rpa_status resident_plan(rpa_ctx* c, int nsys, rpa_ctx::ResidentPlan** ou
         pl.known = true;
       }
       if (pl.sh.G == 0) continue;
-      if (!best || nsys <= pl.sh.clusters) best = &pl;
+      const long long quarters = sizeof(T) == 4 && pl.sh.G == 2 ? 6 : 9;
+      const bool fits = 4LL * n <= quarters * pl.sh.clusters;
+      // fewer systems than n might take this size instead
+      if (by_count && best && !fits) *by_count = true;
+      if (!best || fits) best = &pl;
     }
     if (!best) return RPA_OK;
+    if (by_count && *by_count) return RPA_OK;
     if (!best->tables) CKS(resident_tables<T>(c, *best));
     if (best->sh.G) {
       *out = best;
@@ -1095,11 +1113,23 @@ static rpa_status resident_loop(rpa_ctx* c, const CocgView<T>& cv, rpa_ctx::Resi
 // forms the projector coefficients of r, then iterates the fused kernels.  With cont, the
 // recurrence continues from the direction kept in p (and its projector coefficients in cp)
 // with the beta each system holds, instead of starting from p = r.
+// nact: the number of active systems where the caller knows it, else -1.
 template <typename T>
-static rpa_status cocg_loop(rpa_ctx* c, const CocgView<T>& cv_all, int maxit, bool cont = false) {
+static rpa_status cocg_loop(rpa_ctx* c, const CocgView<T>& cv_all, int maxit, bool cont = false,
+                            int nact = -1) {
   int cnt[kNumStatus];
   rpa_ctx::ResidentPlan* pl = nullptr;
-  CKS(resident_plan<T>(c, cv_all.nsys, &pl));
+  if (sizeof(T) == 4) {
+    CKS(resident_plan<T>(c, cv_all.nsys, &pl));
+  } else {
+    bool by_count = nact < 0;  // counted only where the choice may depend on it
+    if (by_count) CKS(resident_plan<T>(c, cv_all.nsys, &pl, &by_count));
+    if (by_count) {
+      CKS(counts(c, cv_all.nsys, cnt, false));
+      nact = cnt[kActive];
+    }
+    if (nact >= 0) CKS(resident_plan<T>(c, nact, &pl));
+  }
   // Launched iterations until at most `tail` systems are active, the resident kernel from there
   // on.  Up to four blocks per system it wins at any number of systems (26^3, 320 systems: 24
   // against 44 ms per chi0; 27 x 25 x 53: 70 against 109 ms).  Larger clusters leave SMs idle
@@ -1235,8 +1265,9 @@ static rpa_status solve_fp64(rpa_ctx* c, int nb, const double* u, const int* act
                                  c->stream)));
   CK(cocg_scalars(S, cv.tiles, cv.part, cv.sysd, cv.sysi, 0, 1 << kActive, c->opt.stern_tol, 0.0,
                   maxit, 0, c->stream));
+  int nact = -1;
   for (int round = 0; round < 60; ++round) {
-    CKS(cocg_loop<double>(c, cv, maxit));
+    CKS(cocg_loop<double>(c, cv, maxit, false, nact));
     int cnt[kNumStatus];
     CKS(counts(c, S, cnt));
     if (cnt[kConverged] == 0) break;
@@ -1247,7 +1278,8 @@ static rpa_status solve_fp64(rpa_ctx* c, int nb, const double* u, const int* act
     CK(cocg_scalars(S, cv.tiles, cv.part, cv.sysd, cv.sysi, 3, 1 << kConverged,
                     c->opt.stern_tol, 0.0, maxit, 50, c->stream));
     CKS(counts(c, S, cnt));
-    if (cnt[kActive] == 0) break;
+    nact = cnt[kActive];
+    if (nact == 0) break;
   }
   CKS(collect_stats(c, S, ss));
   CK((density<double, double>(c->nd, c->ns, nb, c->d64.psi.as<double>(), x, active,

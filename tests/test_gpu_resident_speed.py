@@ -1,0 +1,45 @@
+"""The resident COCG kernel is chosen where it is the faster path: solves of few systems, where
+larger clusters than fit for all systems at a time are needed to use the GPU, against the launched
+iteration (graphs = 1).  Medians of five calls after two."""
+import time
+
+import numpy as np
+import pytest
+
+import paper_2609_16408_gb300 as R
+from tests.test_gpu_resident import context
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # precision, n, radius, vectors, live vectors, tolerance
+    ("fp64", (26, 26, 26), 4, 1, 1, 1e-3),
+    ("fp64", (26, 26, 26), 6, 1, 1, 1e-3),
+    ("fp64", (26, 26, 26), 6, 20, 1, 1e-8),  # a wave of 320 systems, 16 of them active
+    ("fp64", (30, 30, 30), 6, 1, 1, 1e-3),
+    ("fp64", (30, 30, 30), 6, 1, 1, 1e-8),
+    ("fp64", (23, 23, 23), 6, 3, 3, 1e-3),
+    ("mixed", (30, 30, 30), 6, 3, 3, 1e-4),
+    ("mixed", (36, 36, 36), 6, 1, 1, 1e-4),
+]
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: f"{c[0]}-{c[1][0]}-r{c[2]}-{c[4]}of{c[3]}-{c[5]:g}")
+def test_resident_not_slower_than_launched(case):
+    prec, n, radius, cnt, live, tol = case
+    u = np.random.default_rng(3).standard_normal((cnt, int(np.prod(n))))
+    u[live:] = 0.0
+    om = np.geomspace(0.05, 20.0, cnt) if live > 1 else np.full(cnt, 0.3)
+    t = {}
+    for graphs in (2, 1):
+        c, _ = context(n, (0, 0, 0), radius, 16, 8, 11, precision=prec, stern_tol=tol,
+                       graphs=graphs)
+        x = []
+        for _ in range(7):
+            t0 = time.perf_counter()
+            R.rpa_chi0(c.ctx, om, u, 16)
+            x.append(time.perf_counter() - t0)
+        t[graphs] = sorted(x[2:])[2]
+        c.close()
+    print(f"resident {1e3 * t[2]:.2f} ms, launched {1e3 * t[1]:.2f} ms")
+    assert t[2] <= t[1]
