@@ -123,16 +123,18 @@ struct rpa_ctx {
   long long loop_no = 0;
   int prof_cpx_bytes = 0;
   // resident COCG (cocg_resident.cu) per COCG precision (FP32, FP64) and cluster size 2^i:
-  // shape (known once asked for) and projector tables (built on first use, dropped with the
-  // projectors); h_*: the internal projector groups on the host
+  // shape (known once asked for, for a number of projector groups) and projector tables (built on
+  // first use, dropped with the projectors; no_room: they do not fit); h_*: the internal
+  // projector groups on the host
   struct ResidentPlan {
-    bool known = false, tables = false;
+    bool known = false, tables = false, no_room = false;
     rpa::ResidentShape sh;
-    rpa::DevBuf roff, rstep, gslot, gchi, goff, groups, lwarp, lkey, lchi, gmask;
+    rpa::DevBuf index, gchi, lchi;  // index: the integer tables, at the offsets that follow
+    size_t o_roff = 0, o_rstep = 0, o_goff = 0, o_groups = 0, o_lwarp = 0, o_gmask = 0, o_gslot = 0,
+           o_lkey = 0;
   };
   ResidentPlan resident[2][5];
   std::vector<int> h_goff, h_gidx;
-  std::vector<double> h_gchi;
   // non-fatal outcome of the current call (results are still written): RPA_ENOCONV or
   // RPA_EBREAKDOWN (the more severe is kept), with its reason
   rpa_status soft = RPA_OK;
@@ -894,114 +896,169 @@ static rpa_status run_loop_graph(rpa_ctx* c, const CocgView<T>& cv, const FusedB
   return RPA_OK;
 }
 
-// Projector tables of a resident plan: the internal groups' entries by block of the cluster.
+// Projector tables of a resident plan: the internal groups' entries by block of the cluster (see
+// ResidentProj).  They are built anew for every set of projectors, so a call that sets them pays
+// for it: the host sorts by counting and places indices only, and the device gathers the values
+// (32 atoms on 26 x 52 x 52, 125,000 entries: 1.8 ms for the first solve on top of a later one; with
+// sorted entries and their values 9.5).
 template <typename T>
 static rpa_status resident_tables(rpa_ctx* c, rpa_ctx::ResidentPlan& pl) {
   const ResidentShape& sh = pl.sh;
   const int nx = c->grid.n[0], ny = c->grid.n[1], nz = c->grid.n[2], G = sh.G;
-  const int ng = c->ngroup;
-  // owner brick of every y and z coordinate, and its extents
-  std::vector<int> ry(ny), rz(nz), y0(sh.gy + 1), z0(sh.gz + 1);
-  for (int q = 0; q <= sh.gy; ++q) y0[q] = (int)((long long)q * ny / sh.gy);
-  for (int q = 0; q <= sh.gz; ++q) z0[q] = (int)((long long)q * nz / sh.gz);
-  for (int q = 0; q < sh.gy; ++q)
-    for (int y = y0[q]; y < y0[q + 1]; ++y) ry[y] = q;
-  for (int q = 0; q < sh.gz; ++q)
-    for (int z = z0[q]; z < z0[q + 1]; ++z) rz[z] = q;
-  struct Entry {
-    int layer, slot, group;
-    long long e;
+  const int ng = c->ngroup, nw = sh.threads / 32;
+  const int cap = sh.bym * sh.bzm * sh.pitch;
+  // block and first slot of every grid row
+  struct Row {
+    int rank, slot;
   };
-  std::vector<std::vector<Entry>> grp(G);
-  std::vector<std::vector<unsigned char>> cnt(G, std::vector<unsigned char>(65536, 0));
-  std::vector<unsigned> mask(std::max(ng, 1), 0u);
-  for (int g = 0; g < ng; ++g)
+  std::vector<Row> rows((size_t)ny * nz);
+  for (int rz = 0; rz < sh.gz; ++rz)
+    for (int ry = 0; ry < sh.gy; ++ry) {
+      const int y0 = (int)((long long)ry * ny / sh.gy), y1 = (int)((long long)(ry + 1) * ny / sh.gy);
+      const int z0 = (int)((long long)rz * nz / sh.gz), z1 = (int)((long long)(rz + 1) * nz / sh.gz);
+      for (int z = z0; z < z1; ++z)
+        for (int y = y0; y < y1; ++y)
+          rows[(size_t)z * ny + y] = {ry + sh.gy * rz, ((z - z0) * (y1 - y0) + (y - y0)) * sh.pitch};
+    }
+  // entries of each block in group order; a point's entries are its layers
+  struct Entry {
+    unsigned key;  // group << 16 | slot
+    int e, layer;
+  };
+  const size_t total = c->h_gidx.size();
+  std::vector<std::vector<Entry>> ent(G);
+  for (auto& v : ent) v.reserve(total / G + total / (4 * G) + 64);
+  std::vector<unsigned char> layers((size_t)G * cap, 0);
+  std::vector<int> mask(std::max(ng, 1), 0);
+  for (int g = 0; g < ng; ++g) {
+    int row = 0, x0 = 0;  // the row of the entry before: entries of a group ascend
     for (int e = c->h_goff[g]; e < c->h_goff[g + 1]; ++e) {
-      const int q = c->h_gidx[e], x = q % nx, y = q / nx % ny, z = q / (nx * ny);
-      const int rank = ry[y] + sh.gy * rz[z];
-      const int by = y0[ry[y] + 1] - y0[ry[y]];
-      const int slot = ((z - z0[rz[z]]) * by + (y - y0[ry[y]])) * sh.pitch + x;
-      const int l = cnt[rank][slot];
+      const int q = c->h_gidx[e];
+      if (q < x0 || q >= x0 + nx) {
+        row = q / nx;
+        x0 = row * nx;
+      }
+      const Row& rw = rows[row];
+      const int slot = rw.slot + q - x0;
+      unsigned char& l = layers[(size_t)rw.rank * cap + slot];
       if (l == 255) {  // more groups at a point than the layers count
-        pl.sh.G = 0;
+        pl.no_room = true;
         return RPA_OK;
       }
-      cnt[rank][slot]++;
-      grp[rank].push_back({l, slot, g, e});
-      mask[g] |= 1u << rank;
+      ent[rw.rank].push_back({(unsigned)g << 16 | (unsigned)slot, e, l++});
+      mask[g] |= 1 << rw.rank;
     }
-  const int nw = sh.threads / 32;
-  std::vector<int> roff(1, 0), rstep(1, 0), goff(1, 0), groups, lwarp(1, 0);
+  }
+  const int step = 32, rec = step * res_steps<T>();
+  std::vector<int> roff(1, 0), rstep(1, 0), goff(1, 0), groups, lwarp(1, 0), ge, le;
   std::vector<unsigned short> gslot;
   std::vector<unsigned> lkey;
-  std::vector<T> gchi, lchi;
-  auto put = [&](std::vector<T>& v, long long e) {
-    for (int l = 0; l < kProjChunk; ++l)
-      v.push_back(e < 0 ? (T)0 : (T)c->h_gchi[(size_t)e * kProjChunk + l]);
-  };
+  const size_t most = total + total / 4 + 4096;
+  ge.reserve(most);
+  le.reserve(most);
+  gslot.reserve(most);
+  lkey.reserve(most);
+  std::vector<int> first(cap), pos, fill;
   for (int r = 0; r < G; ++r) {
-    std::vector<Entry>& v = grp[r];
-    for (size_t i = 0; i < v.size();) {  // entries of a group are consecutive
-      size_t j = i;
-      while (j < v.size() && v[j].group == v[i].group) ++j;
-      groups.push_back(v[i].group);
+    const std::vector<Entry>& v = ent[r];
+    // records of one group
+    for (size_t i = 0; i < v.size();) {
+      const unsigned g = v[i].key >> 16;
+      groups.push_back((int)g);
       groups.push_back((int)rstep.size() - 1 - roff.back());
-      while (i < j) {
-        const size_t end = std::min(j, i + 32 * res_steps<T>());
-        for (; i < end; i += 32)
-          for (size_t l = i; l < i + 32; ++l) {
-            gslot.push_back(l < end ? (unsigned short)v[l].slot : 0);
-            put(gchi, l < end ? v[l].e : -1);
-          }
-        i = end;
-        rstep.push_back((int)gslot.size() / 32);
+      while (i < v.size() && v[i].key >> 16 == g) {
+        const size_t at = ge.size();
+        size_t n = 0;
+        while (n < (size_t)rec && i + n < v.size() && v[i + n].key >> 16 == g) ++n;
+        ge.resize(at + (n + step - 1) / step * step, -1);
+        gslot.resize(ge.size(), 0);
+        for (size_t k = 0; k < n; ++k) {
+          ge[at + k] = v[i + k].e;
+          gslot[at + k] = (unsigned short)v[i + k].key;
+        }
+        i += n;
+        rstep.push_back((int)(ge.size() / step));
       }
       groups.push_back((int)rstep.size() - 1 - roff.back());
     }
     goff.push_back((int)groups.size() / 3);
     roff.push_back((int)rstep.size() - 1);
-    if ((roff[r + 1] - roff[r]) * kProjChunk > sh.bym * sh.bzm * sh.pitch) {
-      pl.sh.G = 0;  // the records' sums share the space of w
+    if ((roff[r + 1] - roff[r]) * kProjChunk > cap) {  // the records' sums share the space of w
+      pl.no_room = true;
       return RPA_OK;
     }
-    // runs of slots with about the same number of entries, by layer
-    std::sort(v.begin(), v.end(), [](const Entry& a, const Entry& b) {
-      return a.slot != b.slot ? a.slot < b.slot : a.layer < b.layer;
-    });
-    size_t i = 0;
-    for (int w = 0; w < nw; ++w) {
-      size_t j = w + 1 == nw ? v.size() : std::max(i, v.size() * (size_t)(w + 1) / nw);
-      while (j > i && j < v.size() && v[j].slot == v[j - 1].slot) ++j;
-      std::sort(v.begin() + i, v.begin() + j, [](const Entry& a, const Entry& b) {
-        return a.layer != b.layer ? a.layer < b.layer : a.slot < b.slot;
-      });
-      while (i < j) {
-        const int layer = v[i].layer;
-        for (int l = 0; l < 32; ++l) {
-          const bool in = i < j && v[i].layer == layer;
-          lkey.push_back(in ? (unsigned)v[i].group << 16 | (unsigned)v[i].slot : ~0u);
-          put(lchi, in ? v[i].e : -1);
-          if (in) ++i;
-        }
+    // runs of slots with about the same number of entries, one per warp; in a run, by layer: fill
+    // counts, then holds the next place of, the (warp, layer) lists
+    const unsigned char* const lay = &layers[(size_t)r * cap];
+    int top = 0;
+    for (int s = 0; s < cap; ++s) top = std::max<int>(top, lay[s]);
+    fill.assign((size_t)nw * top + 1, 0);
+    auto each_slot = [&](auto&& fn) {
+      size_t c0 = 0;
+      int w = 0;
+      for (int s = 0; s < cap; ++s) {
+        if (!lay[s]) continue;
+        while (w + 1 < nw && v.size() * (size_t)(w + 1) / nw <= c0) ++w;
+        fn(s, w, (int)c0);
+        c0 += lay[s];
       }
-      lwarp.push_back((int)lkey.size() / 32);
+    };
+    each_slot([&](int s, int w, int c0) {
+      first[s] = c0;
+      for (int l = 0; l < lay[s]; ++l) ++fill[(size_t)w * top + l];
+    });
+    size_t at = lkey.size();
+    for (int w = 0; w < nw; ++w) {
+      for (int l = 0; l < top; ++l) {
+        const int n = fill[(size_t)w * top + l];
+        fill[(size_t)w * top + l] = (int)at;
+        at += (size_t)(n + step - 1) / step * step;
+      }
+      lwarp.push_back((int)(at / step));
+    }
+    lkey.resize(at, ~0u);
+    le.resize(at, -1);
+    pos.resize(v.size());
+    each_slot([&](int s, int w, int c0) {
+      for (int l = 0; l < lay[s]; ++l) pos[c0 + l] = fill[(size_t)w * top + l]++;
+    });
+    for (const Entry& t : v) {
+      const int p = pos[first[t.key & 0xffffu] + t.layer];
+      lkey[p] = t.key;
+      le[p] = t.e;
     }
   }
-  auto up = [&](DevBuf& b, const void* p, size_t bytes) -> rpa_status {
-    CK(b.ensure(std::max<size_t>(bytes, 16)));
-    if (bytes) CK(cudaMemcpyAsync(b.p, p, bytes, cudaMemcpyHostToDevice, c->stream));
-    return RPA_OK;
+  // one copy for the index tables; the values by entry number from the groups' on the device
+  std::vector<unsigned char> blob;
+  auto put = [&](const void* p, size_t bytes) {
+    const size_t o = blob.size();
+    blob.resize(o + (bytes + 15) / 16 * 16);
+    if (bytes) std::memcpy(&blob[o], p, bytes);
+    return o;
   };
-  CKS(up(pl.roff, roff.data(), roff.size() * sizeof(int)));
-  CKS(up(pl.rstep, rstep.data(), rstep.size() * sizeof(int)));
-  CKS(up(pl.gslot, gslot.data(), gslot.size() * sizeof(unsigned short)));
-  CKS(up(pl.gchi, gchi.data(), gchi.size() * sizeof(T)));
-  CKS(up(pl.goff, goff.data(), goff.size() * sizeof(int)));
-  CKS(up(pl.groups, groups.data(), groups.size() * sizeof(int)));
-  CKS(up(pl.lwarp, lwarp.data(), lwarp.size() * sizeof(int)));
-  CKS(up(pl.lkey, lkey.data(), lkey.size() * sizeof(unsigned)));
-  CKS(up(pl.lchi, lchi.data(), lchi.size() * sizeof(T)));
-  CKS(up(pl.gmask, mask.data(), mask.size() * sizeof(unsigned)));
+  blob.reserve(sizeof(int) * (ge.size() + 2 * le.size() + groups.size() + rstep.size() + lwarp.size() +
+                              mask.size() + 4 * G) + 2 * gslot.size() + 1024);
+  pl.o_roff = put(roff.data(), roff.size() * sizeof(int));
+  pl.o_rstep = put(rstep.data(), rstep.size() * sizeof(int));
+  pl.o_goff = put(goff.data(), goff.size() * sizeof(int));
+  pl.o_groups = put(groups.data(), groups.size() * sizeof(int));
+  pl.o_lwarp = put(lwarp.data(), lwarp.size() * sizeof(int));
+  pl.o_gmask = put(mask.data(), mask.size() * sizeof(int));
+  pl.o_gslot = put(gslot.data(), gslot.size() * sizeof(unsigned short));
+  pl.o_lkey = put(lkey.data(), lkey.size() * sizeof(unsigned));
+  const size_t o_ge = put(ge.data(), ge.size() * sizeof(int));
+  const size_t o_le = put(le.data(), le.size() * sizeof(int));
+  const size_t val = sizeof(T) * kProjChunk;
+  CK(pl.index.ensure(std::max<size_t>(blob.size(), 16)));
+  CK(pl.gchi.ensure(std::max<size_t>(ge.size() * val, val)));
+  CK(pl.lchi.ensure(std::max<size_t>(le.size() * val, val)));
+  unsigned char* const ix = pl.index.as<unsigned char>();
+  CK(cudaMemcpyAsync(ix, blob.data(), blob.size(), cudaMemcpyHostToDevice, c->stream));
+  const T* chi = opd<T>(c).g_chi.template as<T>();
+  CK(resident_gather<T>((long long)ge.size(), reinterpret_cast<const int*>(ix + o_ge), chi,
+                        pl.gchi.as<T>(), c->stream));
+  CK(resident_gather<T>((long long)le.size(), reinterpret_cast<const int*>(ix + o_le), chi,
+                        pl.lchi.as<T>(), c->stream));
   CK(cudaStreamSynchronize(c->stream));  // the host arrays go away
   pl.tables = true;
   return RPA_OK;
@@ -1035,7 +1092,7 @@ static rpa_status resident_plan(rpa_ctx* c, int n, rpa_ctx::ResidentPlan** out,
       !resident_supported(c->grid.fd_radius))
     return RPA_OK;
   const int k = sizeof(T) == 4 ? 0 : 1;
-  // a size whose projector tables do not fit drops out (sh.G = 0), and the choice is made again
+  // a size whose projector tables do not fit drops out (no_room), and the choice is made again
   // in the same call, so that it does not depend on the calls before
   for (;;) {
     rpa_ctx::ResidentPlan* best = nullptr;
@@ -1046,7 +1103,7 @@ static rpa_status resident_plan(rpa_ctx* c, int n, rpa_ctx::ResidentPlan** out,
                              c->ngroup, 1 << i, &pl.sh));
         pl.known = true;
       }
-      if (pl.sh.G == 0) continue;
+      if (pl.sh.G == 0 || pl.no_room) continue;
       const long long quarters = sizeof(T) == 4 && pl.sh.G == 2 ? 6 : 9;
       const bool fits = 4LL * n <= quarters * pl.sh.clusters;
       // fewer systems than n might take this size instead
@@ -1056,7 +1113,7 @@ static rpa_status resident_plan(rpa_ctx* c, int n, rpa_ctx::ResidentPlan** out,
     if (!best) return RPA_OK;
     if (by_count && *by_count) return RPA_OK;
     if (!best->tables) CKS(resident_tables<T>(c, *best));
-    if (best->sh.G) {
+    if (best->tables) {
       *out = best;
       return RPA_OK;
     }
@@ -1069,16 +1126,17 @@ static rpa_status resident_loop(rpa_ctx* c, const CocgView<T>& cv, rpa_ctx::Resi
   ResidentProj<T> pj;
   pj.ngroup = c->ngroup;
   pj.coef = opd<T>(c).coef.template as<T>();
-  pj.roff = pl.roff.as<int>();
-  pj.rstep = pl.rstep.as<int>();
-  pj.gslot = pl.gslot.as<unsigned short>();
+  const unsigned char* const ix = pl.index.as<unsigned char>();
+  pj.roff = reinterpret_cast<const int*>(ix + pl.o_roff);
+  pj.rstep = reinterpret_cast<const int*>(ix + pl.o_rstep);
+  pj.gslot = reinterpret_cast<const unsigned short*>(ix + pl.o_gslot);
   pj.gchi = pl.gchi.as<T>();
-  pj.goff = pl.goff.as<int>();
-  pj.groups = pl.groups.as<int>();
-  pj.lwarp = pl.lwarp.as<int>();
-  pj.lkey = pl.lkey.as<unsigned>();
+  pj.goff = reinterpret_cast<const int*>(ix + pl.o_goff);
+  pj.groups = reinterpret_cast<const int*>(ix + pl.o_groups);
+  pj.lwarp = reinterpret_cast<const int*>(ix + pl.o_lwarp);
+  pj.lkey = reinterpret_cast<const unsigned*>(ix + pl.o_lkey);
   pj.lchi = pl.lchi.as<T>();
-  pj.gmask = pl.gmask.as<unsigned>();
+  pj.gmask = reinterpret_cast<const unsigned*>(ix + pl.o_gmask);
   const bool prof = c->opt.profile && c->have_pev && c->prof_stats;
   long long iters = 0;
   auto count = [&](int sign) -> rpa_status {  // iterations of all systems so far
@@ -2242,12 +2300,14 @@ rpa_status rpa_set_projectors(rpa_ctx* c, int ngroups, const int* nnz, const int
     CK(cudaMemcpy(c->p_chi_lo.p, pchi_lo.data(), sizeof(float) * E * kProjChunk, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(c->coef_lo.p, gcoef_lo.data(), sizeof(float) * NG * kProjChunk, cudaMemcpyHostToDevice));
   }
+  for (auto& row : c->resident)
+    for (auto& pl : row) {
+      if (NG != c->ngroup) pl.known = false;  // it sets the shape's shared memory
+      pl.tables = pl.no_room = false;
+    }
   c->ngroup = NG;
-  c->h_goff = goff;
-  c->h_gidx = gidx;
-  c->h_gchi = gchi;
-  for (auto& row : c->resident)  // the number of groups sets the shapes' shared memory
-    for (auto& pl : row) pl.known = pl.tables = false;
+  c->h_goff = std::move(goff);
+  c->h_gidx = std::move(gidx);
   // host copy of the inputs, for lane contexts
   long long nidx = 0, nchi = 0, ngam = 0;
   for (int g = 0; g < ngroups; ++g) {

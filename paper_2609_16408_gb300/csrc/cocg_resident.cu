@@ -1218,7 +1218,27 @@ cudaError_t launch_r(const CocgView<T>& cv, const ResidentShape& sh, const Resid
   return e;
 }
 
+template <typename T>
+__global__ void __launch_bounds__(256) k_resident_gather(long long n, const int* __restrict__ e,
+                                                         const T* __restrict__ chi,
+                                                         T* __restrict__ out) {
+  const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+  if (i >= n) return;
+  T v[kProjChunk] = {0, 0, 0, 0};
+  if (e[i] >= 0) load_chi4(chi + (long long)e[i] * kProjChunk, v);
+#pragma unroll
+  for (int l = 0; l < kProjChunk; ++l) out[i * kProjChunk + l] = v[l];
+}
+
 }  // namespace
+
+template <typename T>
+cudaError_t resident_gather(long long n, const int* e, const T* chi, T* out, cudaStream_t s) {
+  if (n == 0) return cudaSuccess;
+  k_resident_gather<T><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, e, chi, out);
+  note_launch();
+  return cudaGetLastError();
+}
 
 bool resident_supported(int R) { return R == 4 || R == 6; }
 
@@ -1236,6 +1256,9 @@ cudaError_t resident_cocg(const CocgView<T>& cv, const ResidentShape& sh,
                       : launch_r<T, 6>(cv, sh, pj, p_odd, maxit, cont, s);
 }
 
+template cudaError_t resident_gather<float>(long long, const int*, const float*, float*, cudaStream_t);
+template cudaError_t resident_gather<double>(long long, const int*, const double*, double*,
+                                             cudaStream_t);
 template cudaError_t resident_shape<float>(int, int, int, int, int, int, ResidentShape*);
 template cudaError_t resident_shape<double>(int, int, int, int, int, int, ResidentShape*);
 template cudaError_t resident_cocg<float>(const CocgView<float>&, const ResidentShape&,

@@ -46,6 +46,10 @@ struct ResidentProj {
   const unsigned* gmask = nullptr;        // per group: the blocks with entries of it
 };
 
+// out[i] = the four values of entry e[i], zeros where e[i] < 0
+template <typename T>
+cudaError_t resident_gather(long long n, const int* e, const T* chi, T* out, cudaStream_t s);
+
 bool resident_supported(int R);
 // Shape for a grid of nx x ny x nz points and clusters of G blocks (G = 0 in the result if it
 // does not fit).
