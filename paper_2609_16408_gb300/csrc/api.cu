@@ -7,6 +7,7 @@
 // wave individually (early exit, breakdown); their systems are idle from then on.  After the
 // wave, [f(T)]_{11} gives d_j (Algorithm 1).  Interpolation and the E_c sum follow per
 // frequency (Section 3.2).
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -261,6 +262,37 @@ static rpa_status copy_out(rpa_ctx* c, void* dst, const void* src, size_t bytes,
                      where == RPA_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                      c->stream));
   return RPA_OK;
+}
+
+// Whether kernels may use a caller's device array in place: aligned, in this context's device
+// memory, and inside one allocation.  Anything else (another GPU's memory, an odd address, an
+// array that is too short) goes through a copy, which takes it or refuses it.
+static bool usable_in_place(const rpa_ctx* c, const void* p, size_t bytes) {
+  if (reinterpret_cast<uintptr_t>(p) % sizeof(double) != 0) return false;
+  using Query = CUresult (*)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+  static const Query query = []() -> Query {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult st;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault,
+                                         &st) != cudaSuccess ||
+        st != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    return reinterpret_cast<Query>(f);
+  }();
+  if (!query) return false;
+  // unknown addresses give zeros
+  CUpointer_attribute at[4] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL,
+                               CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  unsigned int type = 0;
+  int device = -1;
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  void* out[4] = {&type, &device, &base, &size};
+  const CUdeviceptr q = reinterpret_cast<CUdeviceptr>(p);
+  return query(4, at, out, q) == CUDA_SUCCESS && type == CU_MEMORYTYPE_DEVICE &&
+         device == c->device && q >= base && size >= bytes && q - base <= size - bytes;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -2527,23 +2559,25 @@ rpa_status rpa_interpolate(rpa_ctx* c, const double* d_coarse, double* d_fine, d
   if (!c->have_freq) return fail(c, RPA_ESTATE, "no frequencies set");
   CK(cudaSetDevice(c->device));
   const long long P = num_probes(c);
+  // arrays on the device in place where the kernels may use them, else copies as for the host
+  const size_t cbytes = sizeof(double) * c->nw * P, fbytes = sizeof(double) * c->nw * c->nd;
   const bool dev = where == RPA_DEVICE;
-  CK(c->itec.ensure(sizeof(double)));
-  double* fine = d_fine;
+  const bool co_here = dev && usable_in_place(c, d_coarse, cbytes);
+  const bool fi_here = dev && d_fine && usable_in_place(c, d_fine, fbytes);
+  const bool ec_here = dev && ec && usable_in_place(c, ec, sizeof(double));
   const double* coarse = d_coarse;
-  if (!dev) {
-    CK(c->itco.ensure(sizeof(double) * c->nw * P));
-    CKS(copy_in(c, c->itco.p, d_coarse, sizeof(double) * c->nw * P, where));
+  if (!co_here) {
+    CK(c->itco.ensure(cbytes));
+    CKS(copy_in(c, c->itco.p, d_coarse, cbytes, where));
     coarse = c->itco.as<double>();
   }
-  if (!dev || !d_fine) {
-    CK(c->itfi.ensure(sizeof(double) * c->nw * c->nd));
-    fine = c->itfi.as<double>();
-  }
-  double* ecd = dev && ec ? ec : c->itec.as<double>();
+  if (!fi_here) CK(c->itfi.ensure(fbytes));
+  if (!ec_here) CK(c->itec.ensure(sizeof(double)));
+  double* const fine = fi_here ? d_fine : c->itfi.as<double>();
+  double* const ecd = ec_here ? ec : c->itec.as<double>();
   CKS(interpolate_dev(c, coarse, fine, ecd));
-  if (!dev && d_fine) CKS(copy_out(c, d_fine, fine, sizeof(double) * c->nw * c->nd, where));
-  if (!dev && ec) CKS(copy_out(c, ec, ecd, sizeof(double), where));
+  if (!fi_here && d_fine) CKS(copy_out(c, d_fine, fine, fbytes, where));
+  if (!ec_here && ec) CKS(copy_out(c, ec, ecd, sizeof(double), where));
   CK(cudaStreamSynchronize(c->stream));
   return RPA_OK;
 }
