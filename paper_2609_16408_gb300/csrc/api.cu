@@ -83,9 +83,12 @@ struct rpa_ctx {
   DevBuf lam[3];
   // interpolation operators (transposed, coarse x fine) per axis
   DevBuf interpWt[3], interpTi[3], interpTw[3], cnodes_d[3];
-  // interpolation workspace: coarse and fine arrays of calls on host data, the two
-  // intermediate arrays, partial sums and E_c
+  // interpolation workspace: coarse and fine arrays of calls on data that is not used in place, the
+  // two intermediate arrays, partial sums and E_c; kept between calls up to kInterpKeep bytes
   DevBuf itco, itfi, it1, it2, itpart, itec;
+  size_t interp_bytes() const {
+    return itco.bytes + itfi.bytes + it1.bytes + it2.bytes + itpart.bytes + itec.bytes;
+  }
   std::vector<long long> cnodes[3];
   int interp_built = -1, stride_built[3] = {0, 0, 0};
   // wave workspace
@@ -440,6 +443,7 @@ static int choose_batch(rpa_ctx* c, long long count) {
   if (nb <= 0) {
     size_t fr = 0, tot = 0;
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) fr = (size_t)8 << 30;
+    fr += c->interp_bytes();  // a wave is as large after an interpolation as before it
     const size_t avail = (size_t)(0.55 * c->mem_share * (double)fr);
     nb = (int)std::max<size_t>(1, avail / std::max<size_t>(1, per_probe_bytes(c)));
     nb = std::min(nb, 512);
@@ -1990,6 +1994,18 @@ static long long num_probes(rpa_ctx* c) {
   return P;
 }
 
+// Gives the interpolation workspace back at the end of a call that needed more than kInterpKeep
+// (ten frequencies on 52^3: 8 MB, 20 with the arrays of a call on host data), so that what is kept
+// is small next to a wave.
+constexpr size_t kInterpKeep = (size_t)64 << 20;
+struct InterpTrim {
+  rpa_ctx* c;
+  ~InterpTrim() {
+    if (c->interp_bytes() <= kInterpKeep) return;
+    for (DevBuf* b : {&c->itco, &c->itfi, &c->it1, &c->it2, &c->itpart, &c->itec}) b->release();
+  }
+};
+
 // d_coarse (device, nw x P) -> d_fine (device, nw x N_d) and E_c (device scalar); queued on the
 // context's stream.  d_coarse is read only by the first of the passes, d_fine written by the last.
 static rpa_status interpolate_dev(rpa_ctx* c, const double* dco, double* dfi, double* ec_dev) {
@@ -2566,6 +2582,7 @@ rpa_status rpa_interpolate(rpa_ctx* c, const double* d_coarse, double* d_fine, d
   const bool fi_here = dev && d_fine && usable_in_place(c, d_fine, fbytes);
   const bool ec_here = dev && ec && usable_in_place(c, ec, sizeof(double));
   const double* coarse = d_coarse;
+  const InterpTrim trim{c};
   if (!co_here) {
     CK(c->itco.ensure(cbytes));
     CKS(copy_in(c, c->itco.p, d_coarse, cbytes, where));
@@ -2737,6 +2754,7 @@ rpa_status rpa_energy_density(rpa_ctx* c, double* d_coarse, double* d_fine, doub
   CK(dfi.ensure(sizeof(double) * c->nw * c->nd));
   CK(ecd.ensure(sizeof(double)));
   CK(cudaMemcpyAsync(dco.p, dh.data(), sizeof(double) * count, cudaMemcpyHostToDevice, c->stream));
+  const InterpTrim trim{c};
   CKS(interpolate_dev(c, dco.as<double>(), dfi.as<double>(), ecd.as<double>()));
   if (d_coarse) CKS(copy_out(c, d_coarse, dco.p, sizeof(double) * count, where));
   if (d_fine) CKS(copy_out(c, d_fine, dfi.p, sizeof(double) * c->nw * c->nd, where));
