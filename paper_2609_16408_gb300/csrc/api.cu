@@ -417,13 +417,20 @@ static int gram_chunks(long long nd) {
   return (int)std::max<long long>(1, std::min<long long>(256, (nd + 4095) / 4096));
 }
 
-// FP64 form: more chunks (of at least 96 points) while the tiles of nb probe-points would leave
-// the GPU idle
-static int gram_chunks64(long long nd, int ns, int nb) {
+// FP64 form: more chunks (of at least 96 points) where the tiles of one probe-point would leave the
+// GPU idle.  By grid and states alone: the chunks set the order of the sums, so that a probe-point's
+// guess is the same to the bit alone, within a wave and from rpa_galerkin.  kGramBlocks: four
+// blocks on each of 152 SMs, a number of its own for the same reason.  (Eight states on 12^3, one
+// probe-point: 484 us in one chunk, 6 in 18.)
+constexpr int kGramBlocks = 608;
+static int gram_chunks64(long long nd, int ns) {
   const int ts = ns <= 8 ? 8 : 16, nt = (ns + ts - 1) / ts;
-  const long long tiles = (long long)nb * nt * (nt + 1) / 2;
-  const long long want = std::min<long long>((nd + 95) / 96, (608 + tiles - 1) / tiles);
+  const long long tiles = (long long)nt * (nt + 1) / 2;
+  const long long want = std::min<long long>((nd + 95) / 96, (kGramBlocks + tiles - 1) / tiles);
   return (int)std::min<long long>(256, std::max<long long>(gram_chunks(nd), want));
+}
+static int gram_chunks_of(const rpa_ctx* c) {
+  return c->opt.precision == RPA_FP64 ? gram_chunks64(c->nd, c->ns) : gram_chunks(c->nd);
 }
 
 static size_t per_probe_bytes(const rpa_ctx* c) {
@@ -433,7 +440,7 @@ static size_t per_probe_bytes(const rpa_ctx* c) {
     b += (size_t)ns * nd * sizeof(float4) + (size_t)nd * sizeof(float2);
   b += (size_t)(c->opt.lanczos_max + 1) * nd * 8 + (size_t)nd * 8 * 5 + (size_t)nd * 4 * 3;
   b += (size_t)ns * part_stride(c) * 4 * 8 + (size_t)ns * (kSysD * 8 + kSysI * 4);
-  b += (size_t)ns * ns * (gram_chunks(nd) * 8 + 16);
+  b += (size_t)ns * ns * (gram_chunks_of(c) * 8 + 16);
   b += (size_t)ns * std::max(1, c->ngroup) * kProjChunk * 16 * 3;
   return b;
 }
@@ -483,12 +490,7 @@ static rpa_status ensure_workspace(rpa_ctx* c, int nb) {
   CK(c->part.ensure(sizeof(double) * S * part_stride(c) * 4));
   CK(c->sysd.ensure(sizeof(double) * S * kSysD));
   CK(c->sysi.ensure(sizeof(int) * S * kSysI));
-  // a wave may hold fewer probe-points than nb, with more chunks each
-  size_t gchunks = (size_t)nb * gram_chunks(nd);
-  if (c->opt.precision == RPA_FP64)
-    for (int b = 1; b <= nb; ++b)
-      gchunks = std::max(gchunks, (size_t)b * gram_chunks64(nd, c->ns, b));
-  CK(c->gpart.ensure(sizeof(double) * gchunks * c->ns * c->ns));
+  CK(c->gpart.ensure(sizeof(double) * nb * gram_chunks_of(c) * c->ns * c->ns));
   CK(c->cmat.ensure(cb * nb * c->ns * c->ns));
   CK(c->probe_d.ensure(sizeof(long long) * nb));
   CK(c->pomega_d.ensure(sizeof(double) * nb));
@@ -1352,7 +1354,7 @@ static rpa_status solve_fp64(rpa_ctx* c, int nb, const double* u, const int* act
   CocgView<double> cv = make_view<double>(c, nb, u, x, r, p, w);
   CK(galerkin_guess<double>(c->nd, c->ns, nb, c->d64.psi.as<double>(), c->eps_d.as<double>(),
                             c->pomega_d.as<double>(), u, active, c->dV, c->gpart.as<double>(),
-                            gram_chunks64(c->nd, c->ns, nb), c->cmat.as<cpx<double>>(), x, c->stream));
+                            gram_chunks_of(c), c->cmat.as<cpx<double>>(), x, c->stream));
   CK(set_status(S, c->ns, active, kActive, c->sysi.as<int>(), c->stream));
   CK(proj_dots<double>(cv.nl, c->nd, S, x, cv.sysi, 1 << kActive, cv.cdot, c->stream));
   CK((cocg_resid<double, double>(cv, x, r, p, 1 << kActive, nullptr, nullptr, nullptr,
@@ -1398,7 +1400,7 @@ static rpa_status solve_mixed(rpa_ctx* c, int nb, const float* u32, const int* a
   CocgView<float> cv = make_view<float>(c, nb, u32, x, r, p, w);
   CK(galerkin_guess_tc(c->nd, c->ns, nb, c->d32.psi.as<float>(), c->eps_d.as<double>(),
                        c->pomega_d.as<double>(), u32, active, c->dV, c->gpart.as<double>(),
-                       gram_chunks(c->nd), c->cmat.as<cpx<float>>(), x, c->flags_d.as<int>() + 2,
+                       gram_chunks_of(c), c->cmat.as<cpx<float>>(), x, c->flags_d.as<int>() + 2,
                        c->stream, c->opt.precision == RPA_MIXED_BF16,
                        c->opt.debug_expire_waits));
   CK(set_status(S, c->ns, active, kActive, c->sysi.as<int>(), c->stream));
@@ -2909,7 +2911,7 @@ rpa_status rpa_galerkin(rpa_ctx* c, int count, const double* omega, const double
       CK(convert_d2f(c->u64.as<double>(), c->u32.as<float>(), (long long)nb * nd, c->stream));
       CK(galerkin_guess_tc(nd, c->ns, nb, c->d32.psi.as<float>(), c->eps_d.as<double>(),
                            c->pomega_d.as<double>(), c->u32.as<float>(), c->active_d.as<int>(),
-                           c->dV, c->gpart.as<double>(), gram_chunks(nd),
+                           c->dV, c->gpart.as<double>(), gram_chunks_of(c),
                            c->cmat.as<cpx<float>>(), c->x.as<cpx<float>>(),
                            c->flags_d.as<int>() + 2, c->stream,
                            c->opt.precision == RPA_MIXED_BF16, c->opt.debug_expire_waits));
@@ -2918,7 +2920,7 @@ rpa_status rpa_galerkin(rpa_ctx* c, int count, const double* omega, const double
       CK(galerkin_guess<double>(nd, c->ns, nb, c->d64.psi.as<double>(), c->eps_d.as<double>(),
                                 c->pomega_d.as<double>(), c->u64.as<double>(),
                                 c->active_d.as<int>(), c->dV, c->gpart.as<double>(),
-                                gram_chunks(nd), c->cmat.as<cpx<double>>(),
+                                gram_chunks_of(c), c->cmat.as<cpx<double>>(),
                                 xo.as<cpx<double>>(), c->stream));
     }
     CKS(copy_out(c, x0 + 2 * (long long)s0 * c->ns * nd, xo.p, sizeof(cpx<double>) * n, where));
