@@ -231,6 +231,74 @@ def oracle_error(R, context, wl, om, w, probes, d_ref, P, nd, natom):
     return out
 
 
+def tiling(t):
+    if t <= -101:
+        return (f"bands of {-100 - t} full x rows, two x points per thread, 3-stage "
+                "cp.async pipeline")
+    if t == -7:
+        return "whole COCG loop in one kernel, a cluster per system"
+    if t == -6:
+        return "two-point kernel on packed full rows"
+    if t in (-3, -4):
+        return (f"64 x 8 tiles, two x points per thread, z window in a shared-memory ring, "
+                f"{1 if t == -3 else 2} centre-plane buffer(s)")
+    return (f"{t} full x rows per block" if t > 0
+            else ("64 x 8 tiles, two x points per thread" if t == -2 else "32 x 8 column tiles"))
+
+
+def cocg_roofline(ks, kb, kl, tile_rows, tile_tail, phase_s, precision_bytes, nd, pk):
+    """Roofline of the dominant launched COCG kernel, from the sampled chunks alone, and the
+    resident kernel by itself (its own slot, every launch timed): its share of the COCG phase and
+    the bytes of its vector passes over global memory, which do not bound it.  Without launched
+    iterations the roofline entry is the resident kernel's."""
+    resident = None
+    if kl[7] > 0:
+        resident = dict(kernel="k_cocg_resident", bound=RESIDENT_BOUND[precision_bytes],
+                        launches=int(kl[7]), seconds=float(ks[7]),
+                        ms_per_launch=float(1e3 * ks[7] / kl[7]), global_bytes=float(kb[7]),
+                        global_gbs=float(kb[7] / ks[7] / 1e9), cocg_share=float(ks[7] / phase_s))
+    if sum(ks[:5]) == 0 and resident:
+        return dict(bound=resident["bound"], kernel=resident["kernel"],
+                    achieved=resident["global_gbs"], peak=pk["hbm_gbs"], unit="GB/s",
+                    frac=resident["global_gbs"] / pk["hbm_gbs"], traffic=None,
+                    algorithmic_bytes_per_launch=float(kb[7] / kl[7]),
+                    peak_src=pk["src"] + " (burst copy)", launches=int(kl[7]),
+                    seconds=float(ks[7]), algorithmic_bytes=float(kb[7]),
+                    cocg_share=resident["cocg_share"]), resident
+    hname = ("k_dirmatvec_band" if tile_rows <= -101
+             else "k_dirmatvec_rows" if tile_rows > 0
+             else "k_dirmatvec_x2p" if tile_rows == -6
+             else ("k_dirmatvec_x2" if tile_rows in (-2, -3, -4) else "k_dirmatvec"))
+    names = ["proj_dots", hname, "k_scalars", "k_update_dots", "none"]
+    dom = 1 if ks[1] >= ks[3] else 3
+    achieved = kb[dom] / ks[dom] / 1e9 if ks[dom] > 0 else 0.0
+    # DRAM traffic per launch from the committed ncu capture (dram__bytes_read + write of one
+    # launch, divided by the systems active in that launch), scaled to this run's average
+    # number of active systems per launch; null once the kernel sources have changed.
+    traffic = None
+    tr_path = os.path.join(ROOT, "profiles", "traffic.json")
+    if os.path.exists(tr_path) and kl[dom] > 0:
+        tj = json.load(open(tr_path)).get(names[dom])
+        if tj and tj.get("source_sha") == kernel_source_sha(names[dom]):
+            alg_per_sys = {1: 4, 3: 6}[dom] * 2 * precision_bytes * nd
+            sys_per_launch = kb[dom] / alg_per_sys / kl[dom]
+            # per-system bytes of the captured grid, scaled to this grid's point count
+            scale = nd / tj.get("grid_points", nd)
+            traffic = tj["dram_bytes_per_system"] * scale * sys_per_launch
+    return dict(bound="hbm", kernel=names[dom], achieved=achieved, peak=pk["hbm_gbs"],
+                unit="GB/s", frac=achieved / pk["hbm_gbs"], traffic=traffic,
+                algorithmic_bytes_per_launch=float(kb[dom] / max(1, kl[dom])),
+                peak_src=pk["src"] + " (burst copy)",
+                launches=int(kl[dom]), seconds=float(ks[dom]), algorithmic_bytes=float(kb[dom]),
+                # share of the sampled launched COCG kernel time (classes 0-4; slots 5 and 6
+                # split the same time into tail and bulk chunks)
+                cocg_share=float(ks[dom] / max(1e-30, sum(ks[:5])))), resident
+
+
+# what bounds the resident kernel, by bytes of a real value
+RESIDENT_BOUND = {4: "shared-memory latency and cluster barriers", 8: "FP64 pipe"}
+
+
 def run_ours(args, wl):
     import torch
 
@@ -333,54 +401,10 @@ def run_ours(args, wl):
     tile_rows = int(stats[-1].get("tile_rows", 0)) if stats else 0
     tile_tail = int(stats[-1].get("tile_rows_tail", 0)) if stats else 0
 
-    def tiling(t):
-        if t <= -101:
-            return (f"bands of {-100 - t} full x rows, two x points per thread, 3-stage "
-                    "cp.async pipeline")
-        if t == -7:
-            return "whole COCG loop in one kernel, a cluster per system"
-        if t == -6:
-            return "two-point kernel on packed full rows"
-        if t in (-3, -4):
-            return (f"64 x 8 tiles, two x points per thread, z window in a shared-memory ring, "
-                    f"{1 if t == -3 else 2} centre-plane buffer(s)")
-        return (f"{t} full x rows per block" if t > 0
-                else ("64 x 8 tiles, two x points per thread" if t == -2 else "32 x 8 column tiles"))
-    hname = ("k_dirmatvec_band" if tile_rows <= -101
-             else "k_dirmatvec_rows" if tile_rows > 0
-             else "k_dirmatvec_x2p" if tile_rows == -6
-             else "k_cocg_resident" if tile_rows == -7
-             else ("k_dirmatvec_x2" if tile_rows in (-2, -3, -4) else "k_dirmatvec"))
-    names = ["proj_dots", hname, "k_scalars", "k_update_dots", "none"]
-    dom = 1 if ks[1] >= ks[3] else 3
     pk = peaks()
-    achieved = kb[dom] / ks[dom] / 1e9 if ks[dom] > 0 else 0.0
-    # DRAM traffic per launch from the committed ncu capture (dram__bytes_read + write of one
-    # launch, divided by the systems active in that launch), scaled to this run's average
-    # number of active systems per launch; null once the kernel sources have changed.
-    traffic = None
-    tr_path = os.path.join(ROOT, "profiles", "traffic.json")
-    if os.path.exists(tr_path) and kl[dom] > 0:
-        tj = json.load(open(tr_path)).get(names[dom])
-        if tj and tj.get("source_sha") == kernel_source_sha(names[dom]):
-            alg_per_sys = {1: 4, 3: 6}[dom] * 2 * stats[0]["precision_bytes"] * nd
-            sys_per_launch = kb[dom] / alg_per_sys / kl[dom]
-            # per-system bytes of the captured grid, scaled to this grid's point count
-            scale = nd / tj.get("grid_points", nd)
-            traffic = tj["dram_bytes_per_system"] * scale * sys_per_launch
-    both = dom == 1 and tile_tail == -7 and tile_rows != -7
-    if both:  # launches of two kernels in one class: no per-launch traffic
-        traffic = None
-    roofline = dict(bound="hbm", kernel=names[dom] + (" + k_cocg_resident" if both else ""),
-                    achieved=achieved, peak=pk["hbm_gbs"],
-                    unit="GB/s", frac=achieved / pk["hbm_gbs"], traffic=traffic,
-                    algorithmic_bytes_per_launch=float(kb[dom] / max(1, kl[dom])),
-                    peak_src=pk["src"] + " (burst copy)",
-                    launches=int(kl[dom]), seconds=float(ks[dom]),
-                    algorithmic_bytes=float(kb[dom]),
-                    # share of the sampled COCG kernel time (classes 0-4; slots 5 and 6
-                    # split the same time into tail and bulk chunks)
-                    cocg_share=float(ks[dom] / max(1e-30, sum(ks[:5]))))
+    roofline, resident = cocg_roofline(
+        ks, kb, kl, tile_rows, tile_tail, sum(st["seconds_phase"][2] for st in stats),
+        stats[0]["precision_bytes"] if stats else 4, nd, pk)
 
     # FP64 form and mixed form timed on one and the same seeded sample, and the
     # mixed-vs-FP64 error on it
@@ -484,10 +508,11 @@ def run_ours(args, wl):
                     tile_rows=tile_rows, tile_rows_tail=tile_tail, cuda_graphs={0: "off", 1: "chunks of 4 iterations, host-checked",
                                  2: "whole COCG loops (conditional while nodes)"}[args.graphs],
                     h_apply_tiling=(f"{tiling(tile_rows)} (launches over > 32 systems), "
-                                    f"{tiling(tile_tail)} (<= 32 systems)"
+                                    f"{tiling(tile_tail)} "
+                                    + ("(last active systems)" if tile_tail == -7 else "(<= 32 systems)")
                                     + (" autotuned" if args.tile == -1 else " set by --tile")),
                     parallelism=f"probe-points sharded over {world} GPU(s)"),
-        roofline=roofline, cpu_baseline=cpu, e2e=e2e, gpu_launches=int(launches),
+        roofline=roofline, resident=resident, cpu_baseline=cpu, e2e=e2e, gpu_launches=int(launches),
         clocks=clk, fp64_form=fp64,
         ec_full_seconds_est=full_pts / value,
         cocg=dict(mean_iters=tot_iters / max(1, tot_solves), solves=tot_solves,
@@ -497,12 +522,14 @@ def run_ours(args, wl):
                   nonconv_solves=sum(st["nonconv_solves"] for st in stats),
                   breakdown_solves=sum(st["breakdown_solves"] for st in stats),
                   step_statuses=sorted(set(statuses)),
-                  # share of the sampled COCG kernel time in chunks whose launches covered
-                  # at most 32 systems (the latency-bound tail of the slowest solves)
-                  tail_time_fraction=(float(ks[5] / (ks[5] + ks[6]))
+                  # the latency-bound tail of the slowest solves: the resident kernel's share of
+                  # the COCG phase where it finishes the loops, else the share of the sampled
+                  # COCG kernel time in chunks whose launches covered at most 32 systems
+                  tail_time_fraction=(resident["cocg_share"] if resident and tile_rows != -7
+                                      else float(ks[5] / (ks[5] + ks[6]))
                                       if ks[5] + ks[6] > 0 else None),
                   tail_iteration_fraction=(float(kl[5] / (kl[5] + kl[6]))
-                                           if kl[5] + kl[6] > 0 else None)),
+                                           if kl[5] + kl[6] > 0 and tile_tail != -7 else None)),
         oracle_error=oracle_err,
         phases_s=list(np.sum([st["seconds_phase"] for st in stats], axis=0)) if stats else None,
     )

@@ -163,19 +163,23 @@ typedef struct {
   /* with options.profile: per COCG kernel class (0 projector dots, 1 H apply (matvec),
    * 2 scalar steps, 3 x/r update, 4 direction update) the summed event time, the number
    * of launches, and the algorithmic bytes moved (active systems x grid points x bytes per
-   * point; projector data and scalars not counted).  A launch of the resident kernel counts in
-   * class 1, with ten vector passes per system and iteration (what the launched kernels of an
-   * iteration move; it keeps most of them in shared memory).  Slots 5 and 6 of kernel_seconds: the
-   * time of the sampled chunks whose launches covered at most 32 systems (the tail) and
-   * more (the bulk); slots 5 and 6 of kernel_launches: those chunks' iterations */
+   * point; projector data and scalars not counted), of sampled chunks: one loop in four, one
+   * chunk of four iterations in four.  Slots 5 and 6 of kernel_seconds: the time of the sampled
+   * chunks whose launches covered at most 32 systems (the tail) and more (the bulk); slots 5
+   * and 6 of kernel_launches: those chunks' iterations.  Slot 7: the resident kernel, every
+   * launch of it (a launch runs the iterations of a loop, or its last ones): event time,
+   * launches, and the bytes of its vector passes over global memory, most of them in L2 (per
+   * iteration p for the neighbouring blocks, r and x where they are not in shared memory).  It
+   * counts in no other slot; seconds_phase[2] is the time that it and the launched kernels share */
   double kernel_seconds[8];
   long long kernel_launches[8];
   double kernel_bytes[8];
   int precision_bytes;     /* bytes of one real value in the COCG vectors (4 or 8) */
   int tile_rows;           /* tiling the H-apply kernel used for launches over many systems:
                               0 = 32 x 8 column tiles, -2 = 64 x 8 two-point tiles, h > 0 =
-                              full-row tiles of height h, -7 = the resident kernel (one
-                              thread-block cluster runs the whole COCG loop of a system) */
+                              full-row tiles of height h, -7 = no such launch, the resident
+                              kernel alone (one thread-block cluster runs the whole COCG
+                              loop of a system) */
   int tile_rows_tail;      /* the same for launches over at most 32 systems, or for the last
                               active systems (-7) */
   long long nonconv_solves;   /* solves that ended above the tolerance (iteration cap, or

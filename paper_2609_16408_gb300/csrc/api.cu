@@ -1176,14 +1176,17 @@ static rpa_status resident_loop(rpa_ctx* c, const CocgView<T>& cv, rpa_ctx::Resi
   pj.lchi = pl.lchi.as<T>();
   pj.gmask = reinterpret_cast<const unsigned*>(ix + pl.o_gmask);
   const bool prof = c->opt.profile && c->have_pev && c->prof_stats;
-  long long iters = 0;
-  auto count = [&](int sign) -> rpa_status {  // iterations of all systems so far
+  long long iters = 0, live = 0;
+  auto count = [&](int sign) -> rpa_status {  // iterations of all systems so far, active systems
     std::vector<int> si((size_t)cv.nsys * kSysI);
     CK(cudaMemcpyAsync(si.data(), cv.sysi, sizeof(int) * si.size(), cudaMemcpyDeviceToHost,
                        c->stream));
     CK(cudaStreamSynchronize(c->stream));
-    for (int s = 0; s < cv.nsys; ++s)
-      if (si[(size_t)s * kSysI + kStatus] != kIdle) iters += sign * si[(size_t)s * kSysI + kIters];
+    for (int s = 0; s < cv.nsys; ++s) {
+      const int st = si[(size_t)s * kSysI + kStatus];
+      if (st != kIdle) iters += sign * si[(size_t)s * kSysI + kIters];
+      if (sign < 0 && st == kActive) ++live;
+    }
     return RPA_OK;
   };
   if (prof) {
@@ -1197,9 +1200,16 @@ static rpa_status resident_loop(rpa_ctx* c, const CocgView<T>& cv, rpa_ctx::Resi
     float ms = 0.f;
     CK(cudaEventElapsedTime(&ms, c->pev[0], c->pev[1]));
     rpa_stats* st = c->prof_stats;
-    st->kernel_seconds[1] += 1e-3 * ms;
-    st->kernel_launches[1] += 1;
-    st->kernel_bytes[1] += 10.0 * sizeof(cpx<T>) * (double)iters * (double)c->nd;
+    // vector passes over global memory: per iteration p for the neighbours, r and x where they are
+    // not in shared memory; per loop what is loaded at the start and stored at the end
+    const double per_iter = (pl.sh.G > 1 ? 1.0 : 0.0) + (pl.sh.r_res ? 0.0 : 2.0) +
+                            (pl.sh.x_res ? 0.0 : 2.0);
+    const double per_loop = (cont ? 1.0 : 0.0) + (pl.sh.r_res ? 1.0 : 0.0) +
+                            (pl.sh.x_res ? 2.0 : 0.0) + 1.0;
+    st->kernel_seconds[7] += 1e-3 * ms;
+    st->kernel_launches[7] += 1;
+    st->kernel_bytes[7] += (per_iter * (double)iters + per_loop * (double)live) *
+                           (double)sizeof(cpx<T>) * (double)c->nd;
     st->precision_bytes = (int)(sizeof(cpx<T>) / 2);
   }
   return RPA_OK;
@@ -1245,7 +1255,7 @@ static rpa_status cocg_loop(rpa_ctx* c, const CocgView<T>& cv_all, int maxit, bo
     if (whole || cnt[kActive] <= tail) {
       if (c->prof_stats) {
         // tile_rows keeps naming the launches over many systems where there were any
-        if (whole) c->prof_stats->tile_rows = kTileResident;
+        if (c->prof_stats->tile_rows_tail == 0) c->prof_stats->tile_rows = kTileResident;
         c->prof_stats->tile_rows_tail = kTileResident;
       }
       return resident_loop<T>(c, cv_all, *pl, maxit, cont);
