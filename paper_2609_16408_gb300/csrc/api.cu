@@ -1119,8 +1119,8 @@ constexpr long long kResidentMinPoints = 1536;
 // larger size was between 27 % ahead and 5 % behind, at 4.3 behind.  FP32 from one block to two:
 // three halves, where the launched iteration may win (23^3, 96 systems: 6.6 against 6.8 ms, two
 // blocks 4.4); with more systems one block is ahead of it and keeps its sums.
-// n: in FP64 the active systems, since most of a wave may be done (26^3, one live vector of 20: 28.8
-// ms by the systems of the wave, 26.4 launched).
+// n: active systems, not those of the wave, most of which may be done (26^3 in FP64, one live vector
+// of 20: 28.8 ms by the systems of the wave, 26.4 launched).
 template <typename T>
 static rpa_status resident_plan(rpa_ctx* c, int n, rpa_ctx::ResidentPlan** out,
                                 bool* by_count = nullptr) {
@@ -1219,23 +1219,19 @@ static rpa_status resident_loop(rpa_ctx* c, const CocgView<T>& cv, rpa_ctx::Resi
 // forms the projector coefficients of r, then iterates the fused kernels.  With cont, the
 // recurrence continues from the direction kept in p (and its projector coefficients in cp)
 // with the beta each system holds, instead of starting from p = r.
-// nact: the number of active systems where the caller knows it, else -1.
+// nact: the number of active systems by which the cluster size is chosen, or -1 before it is counted.
 template <typename T>
-static rpa_status cocg_loop(rpa_ctx* c, const CocgView<T>& cv_all, int maxit, bool cont = false,
-                            int nact = -1) {
+static rpa_status cocg_loop(rpa_ctx* c, const CocgView<T>& cv_all, int maxit, bool cont,
+                            int* nact) {
   int cnt[kNumStatus];
   rpa_ctx::ResidentPlan* pl = nullptr;
-  if (sizeof(T) == 4) {
-    CKS(resident_plan<T>(c, cv_all.nsys, &pl));
-  } else {
-    bool by_count = nact < 0;  // counted only where the choice may depend on it
-    if (by_count) CKS(resident_plan<T>(c, cv_all.nsys, &pl, &by_count));
-    if (by_count) {
-      CKS(counts(c, cv_all.nsys, cnt, false));
-      nact = cnt[kActive];
-    }
-    if (nact >= 0) CKS(resident_plan<T>(c, nact, &pl));
+  bool by_count = *nact < 0;  // counted only where the choice may depend on it
+  if (by_count) CKS(resident_plan<T>(c, cv_all.nsys, &pl, &by_count));
+  if (by_count) {
+    CKS(counts(c, cv_all.nsys, cnt, false));
+    *nact = cnt[kActive];
   }
+  if (*nact >= 0) CKS(resident_plan<T>(c, *nact, &pl));
   // Launched iterations until at most `tail` systems are active, the resident kernel from there
   // on.  Up to four blocks per system it wins at any number of systems (26^3, 320 systems: 24
   // against 44 ms per chi0; 27 x 25 x 53: 70 against 109 ms).  Larger clusters leave SMs idle
@@ -1373,7 +1369,7 @@ static rpa_status solve_fp64(rpa_ctx* c, int nb, const double* u, const int* act
                   maxit, 0, c->stream));
   int nact = -1;
   for (int round = 0; round < 60; ++round) {
-    CKS(cocg_loop<double>(c, cv, maxit, false, nact));
+    CKS(cocg_loop<double>(c, cv, maxit, false, &nact));
     int cnt[kNumStatus];
     CKS(counts(c, S, cnt));
     if (cnt[kConverged] == 0) break;
@@ -1418,7 +1414,9 @@ static rpa_status solve_mixed(rpa_ctx* c, int nb, const float* u32, const int* a
   CK((cocg_resid<float, float>(cv, x, r, p, 1 << kActive, nullptr, nullptr, nullptr, c->stream)));
   CK(cocg_scalars(S, cv.tiles, cv.part, cv.sysd, cv.sysi, 5, 1 << kActive, tol, itol, maxit, 0,
                   c->stream));
-  CKS(cocg_loop<float>(c, cv, maxit));
+  // the cluster size of the first loop serves the refinement rounds too
+  int nact = -1;
+  CKS(cocg_loop<float>(c, cv, maxit, false, &nact));
   if (c->opt.refine <= 0) {
     CKS(collect_stats(c, S, ss));
     CK((density<float, float>(c->nd, c->ns, nb, c->d32.psi.as<float>(), x, active,
@@ -1465,7 +1463,7 @@ static rpa_status solve_mixed(rpa_ctx* c, int nb, const float* u32, const int* a
     int cnt[kNumStatus];
     CKS(counts(c, S, cnt));
     if (cnt[kActive] == 0) break;
-    CKS(cocg_loop<float>(c, cv, maxit, cont));
+    CKS(cocg_loop<float>(c, cv, maxit, cont, &nact));
     const int corrected = (1 << kConverged) | (1 << kMaxit) | (1 << kBreakdown);
     CK(accumulate_df(c->nd, S, c->sysi.as<int>(), corrected, round, x, x64, 0, c->stream));
     // systems that were final before this round keep status kFinal and are skipped above;

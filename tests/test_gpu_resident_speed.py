@@ -20,6 +20,7 @@ CASES = [
     ("fp64", (30, 30, 30), 6, 1, 1, 1e-8),
     ("fp64", (23, 23, 23), 6, 3, 3, 1e-3),
     ("mixed", (30, 30, 30), 6, 3, 3, 1e-4),
+    ("mixed", (30, 30, 30), 6, 20, 1, 1e-4),
     ("mixed", (36, 36, 36), 6, 1, 1, 1e-4),
 ]
 
