@@ -562,6 +562,7 @@ static CocgView<T> make_view(rpa_ctx* c, int nb, const T* u, cpx<T>* x, cpx<T>* 
   cv.nsys = nb * c->ns;
   cv.ns = c->ns;
   cv.tiles = part_stride(c);
+  cv.nsm = std::max(1, c->nsm);
   cv.psi = o.psi.template as<T>();
   cv.eps = c->eps_d.as<double>();
   cv.omega = c->pomega_d.as<double>();

@@ -30,6 +30,7 @@ struct CocgView {
   NonlocalDev<T> nl;
   long long nd;
   int nsys, ns, tiles;
+  int nsm;               // SMs of the device, for splits that fill it
   const T* psi;          // ns x N_d
   const double* eps;     // ns
   const double* omega;   // per probe slot

@@ -1,7 +1,7 @@
 // True residual r = b - (H - sigma) x of the Sternheimer systems (Eq. 4) with
 // b_n = -psi_n (.) u, in the 2.5-D blocked form of the fused COCG kernels: a block owns a
-// column tile (see tile_of), walks z with the 2R+1 values of its column in registers and the current
-// xy plane (with an R-wide halo) in shared memory, next plane prefetched.  Used for the
+// column tile (see tile_of), walks z with the 2R+1 values of its column in registers and the
+// current xy plane (with an R-wide halo) in shared memory, next plane prefetched.  Used for the
 // initial residual of every solve, the true-residual recheck of the FP64 form and the FP64
 // residual of each refinement round of the mixed form (T = double, low-precision copies of r
 // in TL = float for the next FP32 round).  Partial sums per tile: ||r||^2, ||b||^2 and
@@ -333,9 +333,8 @@ Tile tile_of(int nx, int ny, int nz_chunks, int max_tiles, size_t value) {
 // Planes per block: fewer where the blocks do not fill the GPU, or fill it by a little more than
 // whole waves.  A block loads 2R planes ahead of its first one, about the time of four.
 // FP64, 8 systems on 12^3 (8 blocks): 67 -> 11 us; double-float, 64 systems on 26 x 52 x 52 (384
-// blocks of which 304 run at once): 452 -> 361 us.
-// Two-die GB300: 152 SMs; a wrong count costs time only.
-constexpr int kSMs = 152;
+// blocks of which 304 run at once): 452 -> 361 us.  The split sets the order in which a system's
+// norms are summed, so their last bits depend on the number of systems, as they do in the H apply.
 int z_chunk(int nz, int zchunk, long long blocks, int max_chunks, int slots) {
   int best = zchunk;
   long long best_cost = 0;
@@ -358,7 +357,7 @@ void launch_r(const CocgView<T>& cv, const cpx<T>* x, cpx<T>* r, cpx<T>* pdir, i
   int zchunk = nz <= 64 ? nz : 32, nzc = (nz + zchunk - 1) / zchunk;
   const Tile t = tile_of<R>(nx, ny, nzc, cv.tiles, sizeof(cpx<T>));
   zchunk = z_chunk(nz, zchunk, (long long)t.n * cv.nsys, cv.tiles / t.n,
-                   kSMs * (sizeof(T) == 4 ? 3 : 2) * (kRThreads / ((t.tx * t.ty + 31) / 32 * 32)));
+                   cv.nsm * (sizeof(T) == 4 ? 3 : 2) * (kRThreads / ((t.tx * t.ty + 31) / 32 * 32)));
   nzc = (nz + zchunk - 1) / zchunk;
   const size_t planes = 2 * sizeof(cpx<T>) * (t.tx + 2 * R) * (t.ty + 2 * R);
   size_t cdb = sizeof(cpx<T>) * cv.nl.ngroup * kProjChunk;

@@ -122,7 +122,7 @@ struct Args {
   Stencil<T> st;
   const T* vloc;
   long long nd;
-  int nsys, ns, nb;
+  int ns, nb;
   const double *eps, *omega;
   typename Val<T>::V *x, *r, *p, *p_odd;
   double* sysd;
@@ -255,7 +255,7 @@ __device__ __forceinline__ bool unit(int u, int lane, int lines, int segs, int& 
 __device__ __forceinline__ int warp_id() { return __shfl_sync(0xffffffffu, tid() >> 5, 0); }
 
 // Segments of L outputs of a line of b points, evenly spread, the first at 0 and the last at
-// b - L: outputs that two segments share belong to the first.
+// b - L: outputs that two segments share belong to the second.
 struct Segs {
   int n, num, den;
   __device__ Segs(int b, int L) {
@@ -1176,7 +1176,6 @@ cudaError_t launch_r(const CocgView<T>& cv, const ResidentShape& sh, const Resid
   a.st = cv.st;
   a.vloc = cv.vloc;
   a.nd = cv.nd;
-  a.nsys = cv.nsys;
   a.ns = cv.ns;
   a.nb = cv.nsys / cv.ns;
   a.eps = cv.eps;

@@ -14,8 +14,9 @@ namespace rpa {
 // gpart[b][c][k][n] = sum_{r in chunk c} psi_k(r) psi_n(r) u_b(r), symmetric in k and n: only
 // the tiles on and above the diagonal are formed, and mirrored.  Bound by the FP64 pipe; tiles of
 // TS = 8 or 16 states waste less of it on padding and on the diagonal than 32 (8 states on
-// 12^3, one probe-point: one block of a 32-tile, 484 us; 8-tiles over 18 chunks, 6 us).  The 256 threads are 256 / (TS/2)^2 groups that take the
-// rows of a stage in turn, 2 x 2 outputs per thread.
+// 12^3, one probe-point: one block of a 32-tile, 484 us; 8-tiles over 18 chunks, 6 us).  The
+// 256 threads are 256 / (TS/2)^2 groups that take the rows of a stage in turn, 2 x 2 outputs per
+// thread.
 template <typename T, int TS>
 __global__ void __launch_bounds__(256) k_gram(long long nd, int ns, const T* __restrict__ psi,
                                               const T* __restrict__ u,

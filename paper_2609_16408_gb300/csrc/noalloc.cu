@@ -66,8 +66,9 @@ extern "C" rpa_status rpa_galerkin_noalloc(long long nd, int ns, const double* p
                                            void* cuda_stream) {
   if (nd < 1 || nd >= (1LL << 31) || ns < 1 || ns > 1024 || count < 0 || !(dV > 0.0))
     return RPA_EINVAL;
-  // the projection kernels take point tiles of 64 along gridDim.x (< 2^31 tiles) and state
-  // tiles of 32 along gridDim.y (<= 32 here): every nd and ns accepted above fits
+  // the projection kernels take point tiles of 64 or more along gridDim.x (< 2^31 tiles) and at
+  // most 32 state tiles (of 32, or one of 8 or 16) along gridDim.y: every nd and ns accepted
+  // above fits
   const int nchunk = chunks_for(nd);
   // the coefficient matrix starts on a 256-byte boundary after the Gram partials
   const size_t gram_bytes = (((size_t)nchunk * ns * ns * sizeof(double)) + 255) & ~(size_t)255;

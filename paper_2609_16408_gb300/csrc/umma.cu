@@ -63,12 +63,6 @@ __device__ __forceinline__ void issue_stage_bf16(uint32_t tmem, uint32_t a, uint
   }
 }
 
-__device__ __forceinline__ void put_split(uint8_t* hi, uint8_t* lo, uint32_t off, float v) {
-  const float h = umma::to_tf32(v);
-  *reinterpret_cast<float*>(hi + off) = h;
-  *reinterpret_cast<float*>(lo + off) = umma::to_tf32(v - h);
-}
-
 // four K-adjacent values of one row: a whole 16-byte core-matrix row of each part, so that
 // eight lanes with eight rows write 128 contiguous bytes (one value per lane along K hits one
 // bank eight times)
