@@ -90,7 +90,11 @@ typedef struct {
   int reorth;            /* 1: full reorthogonalisation of the Lanczos basis (2 passes) */
   int stride[3];         /* coarsening factor g per axis (C_g of Section 3.2) */
   int interp;            /* RPA_INTERP_* */
-  int batch;             /* probe-points in flight per wave; 0 = sized from free memory */
+  int batch;             /* probe-points in flight per wave; 0 = sized from free memory.  The
+                            last bits of a probe-point's results may differ with the wave that it
+                            runs in: how the residual and the H apply are split, and the cluster
+                            size of the resident kernel, go by the number of (active) systems.
+                            Its Galerkin guess does not differ */
   int fkind;             /* RPA_F_* (RPA_F_LOG for the correlation energy) */
   int refine;            /* mixed form: FP64 residual refinement rounds after FP32 COCG */
   double inner_tol;      /* mixed form: FP32 COCG relative tolerance per round

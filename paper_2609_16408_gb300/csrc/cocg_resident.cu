@@ -23,10 +23,18 @@
 // reads per axis instead of 2R.  FP32 complex values are one 64-bit register pair and all
 // their arithmetic is packed (fma.rn.f32x2).
 // What bounds it: FP64, the FP64 pipe (1.7 multiply-adds per clock and SM; about 125 per point
-// and iteration); FP32, latency -- 16 warps per SM, phases separated by barriers.  26^3 points in
-// FP32 (clusters of two, 8,788 points per block): 74,000 cycles per iteration, of which the
-// projector entries from L2 25,000, the three stencil parts 24,000, the pointwise phases 11,000,
-// barriers and scalar steps 14,000.
+// and iteration); FP32, latency -- 16 warps per SM, phases separated by barriers; 41 % of the issue
+// slots and 4 TB/s of L2 are used.  Cycles per iteration (with clock reads between the phases):
+//                              26^3 FP32, two blocks   26^3 FP64, four   12^3 FP64, sixteen
+//   direction and update             10,900                35,000              2,550
+//   projector entries, from L2       26,400                86,500                  -
+//   x, z and y parts                 29,700               187,000             13,200
+//   coefficients                      1,400                 2,000                100
+//   sums over the block               2,200                 4,700              2,800
+//   the three cluster barriers        4,300                50,300              3,600
+//   scalar steps                      4,100                 4,200              3,900
+// (26^3 FP64: the bricks of 13 x 13 rows hold unequal numbers of projector entries, and the others
+// wait 43,000 cycles for the fullest.)
 // Every block of a cluster computes alpha, beta and the status from the same partial sums in
 // the same order, so all of them take the same branches; the barriers are the hardware's.
 #include <cooperative_groups.h>
