@@ -1120,8 +1120,8 @@ constexpr long long kResidentMinPoints = 1536;
 // larger size was between 27 % ahead and 5 % behind, at 4.3 behind.  FP32 from one block to two:
 // three halves, where the launched iteration may win (23^3, 96 systems: 6.6 against 6.8 ms, two
 // blocks 4.4); with more systems one block is ahead of it and keeps its sums.
-// n: active systems, not those of the wave, most of which may be done (26^3 in FP64, one live vector
-// of 20: 28.8 ms by the systems of the wave, 26.4 launched).
+// n: the systems that are not done, not those of the wave, most of which may be (26^3 in FP64, one
+// live vector of 20: 28.8 ms by the systems of the wave, 26.4 launched).
 template <typename T>
 static rpa_status resident_plan(rpa_ctx* c, int n, rpa_ctx::ResidentPlan** out,
                                 bool* by_count = nullptr) {
@@ -1220,7 +1220,8 @@ static rpa_status resident_loop(rpa_ctx* c, const CocgView<T>& cv, rpa_ctx::Resi
 // forms the projector coefficients of r, then iterates the fused kernels.  With cont, the
 // recurrence continues from the direction kept in p (and its projector coefficients in cp)
 // with the beta each system holds, instead of starting from p = r.
-// nact: the number of active systems by which the cluster size is chosen, or -1 before it is counted.
+// nact: the number of systems by which the cluster size is chosen, those that are not done, or -1
+// before it is counted.
 template <typename T>
 static rpa_status cocg_loop(rpa_ctx* c, const CocgView<T>& cv_all, int maxit, bool cont,
                             int* nact) {
@@ -1230,7 +1231,8 @@ static rpa_status cocg_loop(rpa_ctx* c, const CocgView<T>& cv_all, int maxit, bo
   if (by_count) CKS(resident_plan<T>(c, cv_all.nsys, &pl, &by_count));
   if (by_count) {
     CKS(counts(c, cv_all.nsys, cnt, false));
-    *nact = cnt[kActive];
+    // FP32: with those whose guess meets the inner tolerance, which refinement rounds take up
+    *nact = cnt[kActive] + (sizeof(T) == 4 ? cnt[kConverged] : 0);
   }
   if (*nact >= 0) CKS(resident_plan<T>(c, *nact, &pl));
   // Launched iterations until at most `tail` systems are active, the resident kernel from there

@@ -314,7 +314,8 @@ __global__ void k_scalars(int nsys, int tiles, int stride, const double* __restr
     si[kIters] = 0;
     si[kRestarts] = 0;
     si[kIterBase] = 0;
-    si[kStatus] = (bn == 0.0 || rn <= inner_tol * bn) ? kConverged : kActive;
+    // a zero right-hand side needs no refinement round; a guess that meets the inner tolerance does
+    si[kStatus] = bn == 0.0 ? kFinal : rn <= inner_tol * bn ? kConverged : kActive;
     if (!isfinite(rn) || !isfinite(bn)) si[kStatus] = kBreakdown;
   }
 }

@@ -29,3 +29,24 @@ def test_calls_do_not_depend_on_earlier_ones(groups, prec, tol):
     first, second = (R.rpa_chi0(c.ctx, np.array([0.7]), u, ns) for _ in range(2))
     c.close()
     assert np.array_equal(first[1], second[1]) and np.array_equal(first[0], second[0])
+
+
+def test_size_counts_systems_that_refinement_takes_up():
+    """A guess that meets the inner tolerance is not done: the rounds that follow run the whole wave, on the
+    cluster size of a whole wave (320 systems on 26^3: clusters of two, no launched iterations)."""
+    n, ns, cnt, h = (26, 26, 26), 16, 20, (0.45, 0.5, 0.4)
+    nd = int(np.prod(n))
+    rng = np.random.default_rng(8)
+    psi, eps = plane_waves(n, h, (0, 0, 0), ns)
+    c = R.Context(n, h, (0, 0, 0), 6)
+    R.rpa_set_potential(c.ctx, -rng.uniform(0.0, 1.5, nd))
+    R.rpa_set_projectors(c.ctx, [])
+    R.rpa_set_occupied(c.ctx, psi, eps)
+    R.rpa_set_frequencies(c.ctx, np.array([0.5, 2.0]), np.array([1.0, 1.0]))
+    R.rpa_set_options(c.ctx, precision="mixed", stern_tol=1e-6, inner_tol=2.0, refine=2, lanczos_max=1,
+                      profile=1)
+    out = R.rpa_probe_density(c.ctx, rng.choice(nd, cnt, replace=False).astype(np.int64),
+                              (np.arange(cnt) % 2).astype(np.int32), allow_nonconv=True)
+    c.close()
+    assert out["stats"]["refine_rounds"] > 0
+    assert out["stats"]["tile_rows"] == out["stats"]["tile_rows_tail"] == -7
