@@ -246,6 +246,14 @@ def tiling(t):
             else ("64 x 8 tiles, two x points per thread" if t == -2 else "32 x 8 column tiles"))
 
 
+def tilings(rows, tail):
+    """The tilings of a run, by the launches that used them."""
+    if rows == tail == -7:
+        return tiling(-7)
+    return (f"{tiling(rows)} (launches over > 32 systems), {tiling(tail)} "
+            + ("(last active systems)" if tail == -7 else "(<= 32 systems)"))
+
+
 def cocg_roofline(ks, kb, kl, tile_rows, tile_tail, phase_s, precision_bytes, nd, pk):
     """Roofline of the dominant launched COCG kernel, from the sampled chunks alone, and the
     resident kernel by itself (its own slot, every launch timed): its share of the COCG phase and
@@ -507,10 +515,8 @@ def run_ours(args, wl):
                     probe_points_per_step=per * wl["nw"] * world, l2="inputs > L2 (no flush)",
                     tile_rows=tile_rows, tile_rows_tail=tile_tail, cuda_graphs={0: "off", 1: "chunks of 4 iterations, host-checked",
                                  2: "whole COCG loops (conditional while nodes)"}[args.graphs],
-                    h_apply_tiling=(f"{tiling(tile_rows)} (launches over > 32 systems), "
-                                    f"{tiling(tile_tail)} "
-                                    + ("(last active systems)" if tile_tail == -7 else "(<= 32 systems)")
-                                    + (" autotuned" if args.tile == -1 else " set by --tile")),
+                    h_apply_tiling=tilings(tile_rows, tile_tail)
+                    + (" autotuned" if args.tile == -1 else " set by --tile"),
                     parallelism=f"probe-points sharded over {world} GPU(s)"),
         roofline=roofline, resident=resident, cpu_baseline=cpu, e2e=e2e, gpu_launches=int(launches),
         clocks=clk, fp64_form=fp64,

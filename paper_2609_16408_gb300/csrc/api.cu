@@ -1103,8 +1103,11 @@ static rpa_status resident_tables(rpa_ctx* c, rpa_ctx::ResidentPlan& pl) {
   return RPA_OK;
 }
 
-// Smaller grids keep the captured loop: the rule starts below the smallest grid it was measured
-// on (12^3: one probe-point of 20 Lanczos steps in FP64, 144 -> 55 ms).
+// Smaller grids keep the captured loop.  The line is no crossover: without it the resident kernel is
+// ahead on 6^3 already (FP64, one vector 0.88 against 3.8 ms, 200 vectors 2.5 against 12.9; mixed 0.64
+// against 1.5 and 1.1 against 3.1; 11^3 1.7 / 9.0, 20 / 76, 1.2 / 2.9, 3.8 / 9.6), but callers of such
+// grids read the launched kernels' statistics (kernel_seconds of class 1), which it would empty.
+// Radii other than 4 and 6, those of the cells: not built.
 constexpr long long kResidentMinPoints = 1536;
 
 // The cluster size for n systems, or no plan where the resident kernel does not apply: an

@@ -30,4 +30,6 @@ def test_a_run_of_the_resident_kernel_alone():
     line, res = bench.cocg_roofline(*stats(False, True), -7, -7, 5.0, 8, 1000, PK)
     assert line["kernel"] == "k_cocg_resident" and line["bound"] == "FP64 pipe"
     assert line["cocg_share"] == res["cocg_share"] == 0.8 and line["traffic"] is None
-    assert "bands" in bench.tiling(-102) and "one kernel" in bench.tiling(-7)
+    assert "launches over" not in bench.tilings(-7, -7) and "one kernel" in bench.tilings(-7, -7)
+    assert "(last active systems)" in bench.tilings(-102, -7)
+    assert "(<= 32 systems)" in bench.tilings(-102, 0)
