@@ -1104,9 +1104,10 @@ static rpa_status resident_tables(rpa_ctx* c, rpa_ctx::ResidentPlan& pl) {
 }
 
 // Smaller grids keep the captured loop.  The line is no crossover: without it the resident kernel is
-// ahead on 6^3 already (FP64, one vector 0.88 against 3.8 ms, 200 vectors 2.5 against 12.9; mixed 0.64
-// against 1.5 and 1.1 against 3.1; 11^3 1.7 / 9.0, 20 / 76, 1.2 / 2.9, 3.8 / 9.6), but callers of such
-// grids read the launched kernels' statistics (kernel_seconds of class 1), which it would empty.
+// ahead on 6^3 already (FP64, one vector 0.88 against 3.8 ms, 200 vectors 2.5 against 12.9; mixed
+// 0.64 against 1.5 and 1.1 against 3.1; 11^3 1.7 / 9.0, 20 / 76, 1.2 / 2.9, 3.8 / 9.6), but callers
+// of such grids read the launched kernels' statistics (kernel_seconds of class 1), which it would
+// empty.
 // Radii other than 4 and 6, those of the cells: not built.
 constexpr long long kResidentMinPoints = 1536;
 
@@ -1245,13 +1246,14 @@ static rpa_status cocg_loop(rpa_ctx* c, const CocgView<T>& cv_all, int maxit, bo
   // hundreds of systems are faster per system; the crossing was measured at about 8 systems
   // per cluster (52^3, 1,280 systems: 393 ms launched throughout, 389 resident throughout, 369 /
   // 360 / 349 / 346 ms handing over at 1 / 2 / 4 / 8 per cluster).  FP64 is bound by the FP64
-  // pipe, which clusters of 16 use on 112 of the SMs only: two systems per cluster there.
+  // pipe, which clusters of 16 use on 112 of the SMs only: two systems per cluster there, nine
+  // quarters at least, for which resident_plan takes that size.
   int tail = 0;
   if (pl) {
     const bool whole = sizeof(T) == 8 ? pl->sh.G <= 8 : pl->sh.G <= 4;
     if (!whole) {
       tail = 1;
-      while (tail < (sizeof(T) == 8 ? 2 : 8) * pl->sh.clusters) tail *= 2;
+      while (4 * tail < (sizeof(T) == 8 ? 9 : 32) * pl->sh.clusters) tail *= 2;
       CKS(counts(c, cv_all.nsys, cnt, false));
     }
     if (whole || cnt[kActive] <= tail) {
